@@ -26,6 +26,7 @@
 
 #include <mutex>
 
+#include "p2g_chunks.cuh"
 #include "p2g_tiles.cuh"
 
 namespace polypic {
@@ -72,6 +73,7 @@ __device__ __forceinline__ void reduce_node(const GridGeom &g, const uint8_t *s_
     // +0 starts the sum, so it is never -0 and the zeros of unused slots
     // leave it unchanged: the same bits as summing the used tiles alone
     float sm = 0.0f, sv = 0.0f;
+    const bool need_m = gm || gv;  // the adjoint's scatter writes no mass
     if (any_live) {  // CTA-uniform: no tile around this one holds particles otherwise
         constexpr int X = tile_x(A), Y = tile_y(A), Z = tile_z(A);
         const int64_t F = kTileFloats;
@@ -86,7 +88,7 @@ __device__ __forceinline__ void reduce_node(const GridGeom &g, const uint8_t *s_
             if (cz.ok[az] && cy.ok[ay] && cx.ok[ax] &&
                 s_live[cz.live[az] + cy.live[ay] + cx.live[ax]]) {
                 const float *src = tile_base + (cz.part[az] + cy.part[ay] + cx.part[ax]);
-                m[c] = __ldg(src + tile_off(A, 0));
+                if (need_m) m[c] = __ldg(src + tile_off(A, 0));
                 v[c] = __ldg(src + tile_off(A, 1));
             }
         }
@@ -257,27 +259,35 @@ static cudaError_t reduce_tiles(const P2GArgs &P, float *gm[3], float *gp[3], fl
     return cudaGetLastError();
 }
 
+// The tile kernel of a phase.  27 modes, the node-by-node affine map and solid
+// phases (a sheet holds its particles in few cells of a block) take the chunk
+// kernel, whose contraction keeps every lane busy; 1, 4 and 8 modes of a fluid
+// have too little contraction to pay for its exchange buffer: 460 us against
+// 408 (4 modes FP32) and 328 against 300 (8 modes FP16) on the fluids of 3.8
+// and 2.6 million particles, where 27 modes FP32 take 674 instead of 855.
+static cudaError_t launch_p2g(const P2GArgs &P, int R, int fmt, cudaStream_t s) {
+    const int grid = (int)(P.nblocks / kP2GWarps);
+    if (P.affine) {  // Eq 12's affine map: FP32 coefficients, 4, 8 or 27 modes
+        if (fmt != POLYPIC_COEFF_F32) return cudaErrorInvalidValue;
+        return R == 4 ? launch_tiles_aff4(P, grid, s) : launch_chunks_aff(P, R, grid, s);
+    }
+    if (fmt == POLYPIC_COEFF_F32)
+        return R == 27 || (P.mass_abs && R > 1) ? launch_chunks_f32(P, R, grid, s)
+                                                : launch_tiles_f32(P, R, grid, s);
+    return R == 27 ? launch_chunks_16(P, fmt, grid, s) : launch_tiles_16(P, R, fmt, grid, s);
+}
+
 cudaError_t p2g_adjoint_scatter(const P2GArgs &P, float *lv[3], bool accumulate, int R,
                                 cudaStream_t s) {
     const int grid = (int)(P.nblocks / kP2GWarps);
-    const cudaError_t e = launch_tiles_adj(P, R, grid, s);
+    const cudaError_t e = R == 27 ? launch_chunks_adj(P, grid, s) : launch_tiles_adj(P, R, grid, s);
     if (e != cudaSuccess) return e;
     return reduce_tiles(P, nullptr, lv, nullptr, 0.0f, nullptr, accumulate, s);
 }
 
 cudaError_t p2g(const P2GArgs &P, float *gm[3], float *gp[3], float *gv[3], float dt,
                 const float gravity[3], int R, int fmt, cudaStream_t s) {
-    const int grid = (int)(P.nblocks / kP2GWarps);
-    cudaError_t e;
-    if (P.affine) {  // Eq 12's affine map: FP32 coefficients, 4, 8 or 27 modes
-        if (fmt != POLYPIC_COEFF_F32) return cudaErrorInvalidValue;
-        e = launch_tiles_aff(P, R, grid, s);
-    } else if (fmt == POLYPIC_COEFF_F32) {
-        // a solid phase (a sheet) crosses a block in few of its cells: lane teams
-        e = P.mass_abs ? launch_tiles_teams(P, R, grid, s) : launch_tiles_f32(P, R, grid, s);
-    } else {
-        e = launch_tiles_16(P, R, fmt, grid, s);
-    }
+    const cudaError_t e = launch_p2g(P, R, fmt, s);
     if (e != cudaSuccess) return e;
     return reduce_tiles(P, gm, gp, gv, dt, gravity, false, s);
 }
@@ -288,8 +298,7 @@ cudaError_t p2g_reduce(const P2GArgs &P, float *gm[3], float *gp[3], bool accumu
 }
 
 cudaError_t p2g_accumulate(const P2GArgs &P, float *gm[3], float *gp[3], int R, cudaStream_t s) {
-    const int grid = (int)(P.nblocks / kP2GWarps);
-    const cudaError_t e = launch_tiles_f32(P, R, grid, s);
+    const cudaError_t e = launch_p2g(P, R, POLYPIC_COEFF_F32, s);
     if (e != cudaSuccess) return e;
     return reduce_tiles(P, gm, gp, nullptr, 0.0f, nullptr, true, s);
 }

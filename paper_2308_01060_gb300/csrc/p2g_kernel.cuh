@@ -224,90 +224,12 @@ __device__ __forceinline__ void affine_linear(const float *st, int lane, float d
     for (int g = 0; g < 3; ++g) cl[g] = c1 * M[0][g] + c2 * M[1][g] + c3 * M[2][g];
 }
 
-// 8 and 27 modes under the map are not separable per axis: every stencil node
-// evaluates s_r(xi) = f_a(xi_x) f_b(xi_y) f_c(xi_z) at xi = M z, with
-// f_2(xi) = xi^2 - kappa xi - mu2 from the particle's own (unmapped) axis
-// constants kappa = dx t (1 - 4t^2), mu2 = dx^2 / 4, and adds
-// mt w(node) sum_r c_r s_r(xi) into the padded footprint (FP32, physical c).
-template <int R, int A>
-__device__ __forceinline__ void accumulate_mapped(const P2GArgs &P, const float *st, int lane,
-                                                  float mt, int shift, float tu, float tv,
-                                                  float tw, const Stencil1D &fu,
-                                                  const Stencil1D &fv, const Stencil1D &fw,
-                                                  Foot &F) {
-    using S = Stage<R, true>;
-    constexpr int D = axis_degrees(R);
-    float M[3][3];
-    affine_inverse<R, A>(st, lane, P.map_dt, M);
-    const float dx = P.dxpow[1], mu2 = 0.25f * P.dxpow[2];
-    // axes u (= A), v, w as x, y, z indices, and each axis's node offsets
-    constexpr int U = A, V = A == 0 ? 1 : 0, Wx = A == 2 ? 1 : 2;
-    const float t3[3] = {tu, tv, tw};
-    float kap[3];   // by x, y, z
-    float Mz[3][3][3];  // [axis u/v/w][node k][component of xi]
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-        const int ax = e == 0 ? U : (e == 1 ? V : Wx);
-        const float t = t3[e];
-        kap[ax] = dx * t * ((1.0f - 2.0f * t) * (1.0f + 2.0f * t));
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float z = ((float)(k - 1) - t) * dx;
-#pragma unroll
-            for (int g = 0; g < 3; ++g) Mz[e][k][g] = M[g][ax] * z;
-        }
-    }
-    float c[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) c[r] = st[(S::kC + r) * 32 + lane];
-#pragma unroll
-    for (int ku = 0; ku < 3; ++ku)
-#pragma unroll
-        for (int kv = 0; kv < 3; ++kv)
-#pragma unroll
-            for (int kw = 0; kw < 3; ++kw) {
-                float f[3][3];  // [axis x/y/z][degree]
-#pragma unroll
-                for (int g = 0; g < 3; ++g) {
-                    const float xi = Mz[0][ku][g] + Mz[1][kv][g] + Mz[2][kw][g];
-                    f[g][0] = 1.0f;
-                    f[g][1] = xi;
-                    f[g][2] = fmaf(xi, xi - kap[g], -mu2);
-                }
-                float Sn = 0.0f;
-#pragma unroll
-                for (int a = 0; a < D; ++a) {
-                    float Sa = 0.0f;
-#pragma unroll
-                    for (int b = 0; b < D; ++b) {
-                        float Sb = 0.0f;
-#pragma unroll
-                        for (int cc = 0; cc < D; ++cc)
-                            if (has_mode(R, a, b, cc))
-                                Sb = fmaf(c[mode_index(a, b, cc)], f[2][cc], Sb);
-                        Sa = fmaf(Sb, f[1][b], Sa);
-                    }
-                    Sn = fmaf(Sa, f[0][a], Sn);
-                }
-                // node ku lands on footprint row ku + shift; both candidate
-                // rows are static indices (the footprint stays in registers)
-                const float w = mt * fu.W[ku] * fv.W[kv] * fw.W[kw];
-                const float wS = w * Sn;
-                F.add(ku, kv, kw, shift ? 0.0f : w, shift ? 0.0f : wS);
-                F.add(ku + 1, kv, kw, shift ? w : 0.0f, shift ? wS : 0.0f);
-            }
-}
-
 template <int R, int FMT, int A, bool ADJ, bool AFF = false>
 __device__ __forceinline__ void accumulate(const P2GArgs &P, const float *st, int lane, float mt,
                                            int shift, const Stencil1D &fu, const Stencil1D &fv,
-                                           const Stencil1D &fw, bool gu, bool gv, bool gw, Foot &F,
-                                           float tu = 0.0f, float tv = 0.0f, float tw = 0.0f) {
+                                           const Stencil1D &fw, bool gu, bool gv, bool gw,
+                                           Foot &F) {
     using S = Stage<R, AFF, FMT>;
-    if constexpr (AFF && R > 4) {
-        accumulate_mapped<R, A>(P, st, lane, mt, shift, tu, tv, tw, fu, fv, fw, F);
-        return;
-    }
     float cl[3] = {0.0f, 0.0f, 0.0f};
     if constexpr (AFF) affine_linear<R, A>(st, lane, P.map_dt, cl);
     constexpr int D = axis_degrees(R);
