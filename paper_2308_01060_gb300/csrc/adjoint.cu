@@ -20,12 +20,20 @@
 // + sum_a sum_abc mu_abc sum_i d/dx_b(G_a G_b G_c) v_ia  (gathered here).
 // P2G adjoint: lc_abc = mt sum_i F_a F_b F_c lmv_ia;  lx_b += mt sum_a sum_i
 // [d/dx_b(W W W) lm_ia + sum_abc c_abc d/dx_b(F_a F_b F_c) lmv_ia].
+#include <type_traits>
+
 #include "adjoint.cuh"
+#include "cp_async.cuh"
 #include "p2g.cuh"
 
 namespace polypic {
 
 constexpr int kAdjThreads = 256;
+// Two CTAs an SM (128 registers) where that spills little: the G2P adjoint of
+// every mode set (27 modes with its scatter 319 -> 306 us on 863 thousand
+// particles) and the P2G adjoint of up to 8 modes (165 -> 130); the P2G adjoint
+// of 27 modes would spill 376 bytes a thread (262 -> 275 us).
+constexpr int p2g_adj_ctas(int R) { return R == 27 ? 1 : 2; }
 template <int A> struct ATile {
     static constexpr int X = A == 0 ? 11 : 10, Y = A == 1 ? 11 : 10, Z = A == 2 ? 7 : 6;
     static constexpr int N = X * Y * Z;
@@ -116,13 +124,17 @@ __device__ __forceinline__ void fit_rows_d(const AxisFac &f, float inv_dx, float
 }
 
 // sum_abc mu_abc sum_i d/dx_b (X_a Y_b Z_c)(i) v(i) for b = x, y, z, with the
-// contraction over x first, then y, then z, streamed over a.
-template <int R, int D>
+// contraction over x first, then y, then z, streamed over a.  A factor and its
+// derivative meet the same operand, so the two run as one packed FP32 FMA (each
+// half rounds as fmaf does).  ZERO2: the degree-2 derivative rows are 0 (the
+// fit's), and their terms are left out: 126 of 648 FMAs of a component.
+template <int R, int D, bool ZERO2, class Mu>
 __device__ __forceinline__ void adj_position(const float (&X)[D][3], const float (&dX)[D][3],
                                              const float (&Y)[D][3], const float (&dY)[D][3],
                                              const float (&Z)[D][3], const float (&dZ)[D][3],
-                                             const float (&v)[3][3][3], const float (&mu)[D][D][D],
-                                             float &Dx, float &Dy, float &Dz) {
+                                             const float (&v)[3][3][3], const Mu &mu, float &Dx,
+                                             float &Dy, float &Dz) {
+    auto bc = [](float f) { return make_float2(f, f); };
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         float U1[3][3], U1d[3][3];  // [ky][kz]
@@ -130,43 +142,59 @@ __device__ __forceinline__ void adj_position(const float (&X)[D][3], const float
         for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
             for (int kz = 0; kz < 3; ++kz) {
-                U1[ky][kz] = fmaf(X[a][0], v[0][ky][kz], fmaf(X[a][1], v[1][ky][kz], X[a][2] * v[2][ky][kz]));
-                U1d[ky][kz] = fmaf(dX[a][0], v[0][ky][kz], fmaf(dX[a][1], v[1][ky][kz], dX[a][2] * v[2][ky][kz]));
+                if (ZERO2 && a == 2) {
+                    U1[ky][kz] = fmaf(X[a][0], v[0][ky][kz], fmaf(X[a][1], v[1][ky][kz], X[a][2] * v[2][ky][kz]));
+                    U1d[ky][kz] = 0.0f;
+                } else {
+                    float2 t = __fmul2_rn(make_float2(X[a][2], dX[a][2]), bc(v[2][ky][kz]));
+                    t = __ffma2_rn(make_float2(X[a][1], dX[a][1]), bc(v[1][ky][kz]), t);
+                    t = __ffma2_rn(make_float2(X[a][0], dX[a][0]), bc(v[0][ky][kz]), t);
+                    U1[ky][kz] = t.x;
+                    U1d[ky][kz] = t.y;
+                }
             }
 #pragma unroll
         for (int b = 0; b < D; ++b) {
-            float U2[3], U2dy[3], U2dx[3];
+            float m[D];
+#pragma unroll
+            for (int c = 0; c < D; ++c) m[c] = has_mode(R, a, b, c) ? mu(a, b, c) : 0.0f;
 #pragma unroll
             for (int kz = 0; kz < 3; ++kz) {
-                U2[kz] = fmaf(Y[b][0], U1[0][kz], fmaf(Y[b][1], U1[1][kz], Y[b][2] * U1[2][kz]));
-                U2dy[kz] = fmaf(dY[b][0], U1[0][kz], fmaf(dY[b][1], U1[1][kz], dY[b][2] * U1[2][kz]));
-                U2dx[kz] = fmaf(Y[b][0], U1d[0][kz], fmaf(Y[b][1], U1d[1][kz], Y[b][2] * U1d[2][kz]));
-            }
-#pragma unroll
-            for (int kz = 0; kz < 3; ++kz) {
-                float M = 0.0f, Md = 0.0f;
+                float2 u;  // U1 contracted with Y_b and dY_b
+                if (ZERO2 && b == 2) {
+                    u = make_float2(fmaf(Y[b][0], U1[0][kz], fmaf(Y[b][1], U1[1][kz], Y[b][2] * U1[2][kz])), 0.0f);
+                } else {
+                    u = __fmul2_rn(make_float2(Y[b][2], dY[b][2]), bc(U1[2][kz]));
+                    u = __ffma2_rn(make_float2(Y[b][1], dY[b][1]), bc(U1[1][kz]), u);
+                    u = __ffma2_rn(make_float2(Y[b][0], dY[b][0]), bc(U1[0][kz]), u);
+                }
+                float2 M = make_float2(0.0f, 0.0f);  // the modes (a, b, *) with Z and dZ
 #pragma unroll
                 for (int c = 0; c < D; ++c)
                     if (has_mode(R, a, b, c)) {
-                        M = fmaf(mu[a][b][c], Z[c][kz], M);
-                        Md = fmaf(mu[a][b][c], dZ[c][kz], Md);
+                        if (ZERO2 && c == 2) M.x = fmaf(m[c], Z[c][kz], M.x);
+                        else M = __ffma2_rn(bc(m[c]), make_float2(Z[c][kz], dZ[c][kz]), M);
                     }
-                Dx = fmaf(M, U2dx[kz], Dx);
-                Dy = fmaf(M, U2dy[kz], Dy);
-                Dz = fmaf(Md, U2[kz], Dz);
+                if (!(ZERO2 && a == 2)) {
+                    const float ux = fmaf(Y[b][0], U1d[0][kz], fmaf(Y[b][1], U1d[1][kz], Y[b][2] * U1d[2][kz]));
+                    Dx = fmaf(M.x, ux, Dx);
+                }
+                if (!(ZERO2 && b == 2)) Dy = fmaf(M.x, u.y, Dy);
+                Dz = fmaf(M.y, u.x, Dz);
             }
         }
     }
 }
 
-// out_abc = sum_i X_a Y_b Z_c v(i) for the modes of the set.
-template <int R, int D>
+// out(r) = sum_i X_a Y_b Z_c v(i) for the modes r = (a, b, c) of the set, handed
+// out degree a by degree a (at most 9 values live).
+template <int R, int D, class Out>
 __device__ __forceinline__ void contract_modes(const float (&X)[D][3], const float (&Y)[D][3],
                                                const float (&Z)[D][3], const float (&v)[3][3][3],
-                                               float (&out)[D][D][D]) {
+                                               const Out &out) {
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        float U1[3][3];
+        float U1[3][3], m[D][D];
 #pragma unroll
         for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
@@ -180,10 +208,9 @@ __device__ __forceinline__ void contract_modes(const float (&X)[D][3], const flo
                 U2[kz] = fmaf(Y[b][0], U1[0][kz], fmaf(Y[b][1], U1[1][kz], Y[b][2] * U1[2][kz]));
 #pragma unroll
             for (int c = 0; c < D; ++c)
-                out[a][b][c] = has_mode(R, a, b, c)
-                                   ? fmaf(Z[c][0], U2[0], fmaf(Z[c][1], U2[1], Z[c][2] * U2[2]))
-                                   : 0.0f;
+                m[b][c] = fmaf(Z[c][0], U2[0], fmaf(Z[c][1], U2[1], Z[c][2] * U2[2]));
         }
+        out(a, m);
     }
 }
 
@@ -243,11 +270,36 @@ __device__ __forceinline__ ParticleAxes particle_axes(const GridGeom &g, float p
     return P;
 }
 
+// ---------------------------------------------------------------- coefficient stages
+// A thread's R coefficients of one component ([mode][thread], its own column
+// only): two stages of shared memory filled by cp.async one component ahead of
+// their use: loaded into registers when a component began, they cost a memory
+// latency each time with 8 warps an SM to hide it.
+template <int R> struct CoeffStage {
+    float *at;      // the thread's column of the stage in use
+    int other = R * kAdjThreads;  // the other stage, from here
+    __device__ __forceinline__ CoeffStage(float *smem) : at(smem + threadIdx.x) {}
+    __device__ __forceinline__ void fill(bool ahead, const float *src, int64_t cnt) {
+        float *to = at + (ahead ? other : 0);
+#pragma unroll
+        for (int r = 0; r < R; ++r, src += cnt) cp_async4(to + r * kAdjThreads, src);
+    }
+    __device__ __forceinline__ void next() {
+        at += other;
+        other = -other;
+    }
+    __device__ __forceinline__ float operator()(int a, int b, int c) const {
+        return at[mode_index(a, b, c) * kAdjThreads];
+    }
+};
+template <int R> constexpr int stage_bytes() { return 2 * R * kAdjThreads * (int)sizeof(float); }
+
 // ---------------------------------------------------------------- G2P adjoint gather
 template <int R, int A>
 __device__ __forceinline__ void g2p_adj_component(const AdjG2PArgs &G, const ParticleAxes &pa,
                                                   const float *tile, int ox, int oy, int oz,
-                                                  uint32_t j, float px_a, float (&lx)[3]) {
+                                                  uint32_t j, float px_a, const CoeffStage<R> &bar,
+                                                  float (&lx)[3]) {
     constexpr int D = axis_degrees(R);
     const Axis &ax = A == 0 ? pa.fce[0] : pa.ctr[0];
     const Axis &ay = A == 1 ? pa.fce[1] : pa.ctr[1];
@@ -271,29 +323,15 @@ __device__ __forceinline__ void g2p_adj_component(const AdjG2PArgs &G, const Par
     const float xn = fmaf(G.dt, c0, px_a);
     const bool clamped = xn < G.g.lo[A] || xn > G.g.hi[A];
     const float lxo = __ldg(G.bar_x[A] + j);
-    // all loads of the component first (read-only path), then the stores:
-    // the loads go out together instead of one per store
-    const int64_t cnt = G.count;
-    const float *__restrict__ bc = G.bar_c + (int64_t)A * R * cnt + j;
-    float *__restrict__ mo = G.mu + (int64_t)A * R * cnt + j;
-    float mu[D][D][D];
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int b = 0; b < D; ++b)
-#pragma unroll
-            for (int c = 0; c < D; ++c)
-                mu[a][b][c] = has_mode(R, a, b, c) ? __ldg(bc + mode_index(a, b, c) * cnt) : 0.0f;
-    if (!clamped) mu[0][0][0] = fmaf(G.dt, lxo, mu[0][0][0]);
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int b = 0; b < D; ++b)
-#pragma unroll
-            for (int c = 0; c < D; ++c)
-                if (has_mode(R, a, b, c)) mo[mode_index(a, b, c) * cnt] = mu[a][b][c];
+    // the effective coefficient adjoint mu is bar c' but for the constant mode,
+    // which also gets the advection's term: only that mode is written for the
+    // scatter, which reads the others where they are (all 27 written and read
+    // again were 560 MB at 863 thousand particles, now 311)
+    const float mu0 = clamped ? bar(0, 0, 0) : fmaf(G.dt, lxo, bar(0, 0, 0));
+    G.mu0[(int64_t)A * G.count + j] = mu0;
+    auto mu = [&](int a, int b, int c) { return a + b + c == 0 ? mu0 : bar(a, b, c); };
     float Dx = 0.0f, Dy = 0.0f, Dz = 0.0f;
-    adj_position<R, D>(X, dX, Y, dY, Z, dZ, v, mu, Dx, Dy, Dz);
+    adj_position<R, D, true>(X, dX, Y, dY, Z, dZ, v, mu, Dx, Dy, Dz);
     lx[0] += Dx;
     lx[1] += Dy;
     lx[2] += Dz;
@@ -301,7 +339,7 @@ __device__ __forceinline__ void g2p_adj_component(const AdjG2PArgs &G, const Par
 }
 
 template <int R>
-__global__ void __launch_bounds__(kAdjThreads) k_g2p_adjoint(AdjG2PArgs G) {
+__global__ void __launch_bounds__(kAdjThreads, 2) k_g2p_adjoint(AdjG2PArgs G) {
     __shared__ float s_tile[kATileFloats];
     const GridGeom &g = G.g;
     const uint32_t tile = blockIdx.x;
@@ -314,7 +352,10 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adjoint(AdjG2PArgs G) {
     stage_tile(g, G.vel, ox, oy, oz, s_tile);
     __syncthreads();
     // software pipeline: the next particle's index and position load while
-    // this one is computed
+    // this one is computed, every component's coefficients one ahead
+    extern __shared__ float s_stage[];
+    CoeffStage<R> bar(s_stage);
+    const int64_t cnt = G.count;
     uint32_t j = jb + threadIdx.x;
     uint32_t pn = j < je ? G.perm[j] : 0u;
     float nx = 0.0f, ny = 0.0f, nz = 0.0f;
@@ -322,27 +363,35 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adjoint(AdjG2PArgs G) {
         nx = G.x[0][pn];
         ny = G.x[1][pn];
         nz = G.x[2][pn];
+        bar.fill(false, G.bar_c + j, cnt);
     }
+    cp_async_commit();
     for (; j < je; j += kAdjThreads) {
         const uint32_t p = pn;
         const float px = nx, py = ny, pz = nz;
-        if (j + kAdjThreads < je) {
-            pn = G.perm[j + kAdjThreads];
+        const uint32_t jn = j + kAdjThreads;
+        if (jn < je) {
+            pn = G.perm[jn];
             nx = G.x[0][pn];
             ny = G.x[1][pn];
             nz = G.x[2][pn];
         }
         const ParticleAxes pa = particle_axes(g, px, py, pz, tx, ty, tz);
         float lx[3] = {0.0f, 0.0f, 0.0f};
-        if (pa.ok) {
-            g2p_adj_component<R, 0>(G, pa, s_tile, ox, oy, oz, j, px, lx);
-            g2p_adj_component<R, 1>(G, pa, s_tile, ox, oy, oz, j, py, lx);
-            g2p_adj_component<R, 2>(G, pa, s_tile, ox, oy, oz, j, pz, lx);
-        } else {
-            atomicOr(G.status, kFlagOutOfDomain);
-            for (int a = 0; a < 3; ++a)
-                for (int r = 0; r < R; ++r) G.mu[((int64_t)a * R + r) * G.count + j] = 0.0f;
-        }
+        auto component = [&](auto axis, float pos) {
+            constexpr int A = decltype(axis)::value;
+            if (A < 2) bar.fill(true, G.bar_c + (int64_t)(A + 1) * R * cnt + j, cnt);
+            else if (jn < je) bar.fill(true, G.bar_c + jn, cnt);
+            cp_async_commit();
+            cp_async_wait<1>();
+            if (pa.ok) g2p_adj_component<R, A>(G, pa, s_tile, ox, oy, oz, j, pos, bar, lx);
+            else G.mu0[(int64_t)A * cnt + j] = 0.0f;
+            bar.next();
+        };
+        component(std::integral_constant<int, 0>{}, px);
+        component(std::integral_constant<int, 1>{}, py);
+        component(std::integral_constant<int, 2>{}, pz);
+        if (!pa.ok) atomicOr(G.status, kFlagOutOfDomain);
         if (G.accumulate) {  // three loads, then three stores
             const float o0 = G.out_x[0][p], o1 = G.out_x[1][p], o2 = G.out_x[2][p];
             lx[0] += o0;
@@ -359,7 +408,7 @@ template <int R, int A>
 __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const ParticleAxes &pa,
                                                   const float *tile_m, const float *tile_v, int ox,
                                                   int oy, int oz, uint32_t p, float mt,
-                                                  float (&lx)[3]) {
+                                                  const CoeffStage<R> &coef, float (&lx)[3]) {
     constexpr int D = axis_degrees(R);
     const Axis &ax = A == 0 ? pa.fce[0] : pa.ctr[0];
     const Axis &ay = A == 1 ? pa.fce[1] : pa.ctr[1];
@@ -370,69 +419,105 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     p2g_rows<D>(fy, Q.dx, Q.inv_dx, Y, dY);
     p2g_rows<D>(fz, Q.dx, Q.inv_dx, Z, dZ);
     const int lx0 = ax.base - ox, ly0 = ay.base - oy, lz0 = az.base - oz;
-    float lmv[3][3][3], lm[3][3][3];
-    read_stencil<A>(tile_v, lx0, ly0, lz0, lmv);
-    read_stencil<A>(tile_m, lx0, ly0, lz0, lm);
     const int64_t cnt = Q.count;
-    // the component's coefficients first (read-only path, all in flight at
-    // once), then the coefficient adjoint and its stores
-    const float *__restrict__ cin = Q.coeff + (int64_t)A * R * cnt + p;
     float *__restrict__ cout = Q.out_c + (int64_t)A * R * cnt + p;
-    float c[D][D][D];
+    float Dx = 0.0f, Dy = 0.0f, Dz = 0.0f;
+    {  // position terms of the mass, through the weights
+        float lm[3][3][3];
+        read_stencil<A>(tile_m, lx0, ly0, lz0, lm);
+        float Wx[1][3], dWx[1][3], Wy[1][3], dWy[1][3], Wz[1][3], dWz[1][3];
 #pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int b = 0; b < D; ++b)
-#pragma unroll
-            for (int cc = 0; cc < D; ++cc)
-                c[a][b][cc] = has_mode(R, a, b, cc) ? __ldg(cin + mode_index(a, b, cc) * cnt) : 0.0f;
-    float lc[D][D][D];
-    contract_modes<R, D>(X, Y, Z, lmv, lc);
-    if (Q.accumulate) {  // the old values, all loaded before the first store
-#pragma unroll
-        for (int a = 0; a < D; ++a)
+        for (int k = 0; k < 3; ++k) {
+            Wx[0][k] = X[0][k]; dWx[0][k] = dX[0][k];
+            Wy[0][k] = Y[0][k]; dWy[0][k] = dY[0][k];
+            Wz[0][k] = Z[0][k]; dWz[0][k] = dZ[0][k];
+        }
+        auto one = [](int, int, int) { return 1.0f; };
+        adj_position<1, 1, false>(Wx, dWx, Wy, dWy, Wz, dWz, lm, one, Dx, Dy, Dz);
+    }
+    float lmv[3][3][3];
+    read_stencil<A>(tile_v, lx0, ly0, lz0, lmv);
+    contract_modes<R, D>(X, Y, Z, lmv, [&](int a, const float (&m)[D][D]) {
+        float old[D][D];
+        if (Q.accumulate) {  // the old values, loaded before the first store
 #pragma unroll
             for (int b = 0; b < D; ++b)
 #pragma unroll
                 for (int cc = 0; cc < D; ++cc)
-                    lc[a][b][cc] = has_mode(R, a, b, cc)
-                                       ? fmaf(mt, lc[a][b][cc], cout[mode_index(a, b, cc) * cnt])
-                                       : 0.0f;
-    } else {
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-#pragma unroll
-            for (int b = 0; b < D; ++b)
-#pragma unroll
-                for (int cc = 0; cc < D; ++cc) lc[a][b][cc] *= mt;
-    }
-#pragma unroll
-    for (int a = 0; a < D; ++a)
+                    old[b][cc] = has_mode(R, a, b, cc) ? cout[mode_index(a, b, cc) * cnt] : 0.0f;
+        }
 #pragma unroll
         for (int b = 0; b < D; ++b)
 #pragma unroll
             for (int cc = 0; cc < D; ++cc)
-                if (has_mode(R, a, b, cc)) cout[mode_index(a, b, cc) * cnt] = lc[a][b][cc];
-    // position terms: momentum through the modes, mass through the weights
-    float Dx = 0.0f, Dy = 0.0f, Dz = 0.0f;
-    adj_position<R, D>(X, dX, Y, dY, Z, dZ, lmv, c, Dx, Dy, Dz);
-    float Wx[1][3], dWx[1][3], Wy[1][3], dWy[1][3], Wz[1][3], dWz[1][3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        Wx[0][k] = X[0][k]; dWx[0][k] = dX[0][k];
-        Wy[0][k] = Y[0][k]; dWy[0][k] = dY[0][k];
-        Wz[0][k] = Z[0][k]; dWz[0][k] = dZ[0][k];
-    }
-    const float one[1][1][1] = {{{1.0f}}};
-    adj_position<1, 1>(Wx, dWx, Wy, dWy, Wz, dWz, lm, one, Dx, Dy, Dz);
+                if (has_mode(R, a, b, cc))
+                    cout[mode_index(a, b, cc) * cnt] =
+                        Q.accumulate ? fmaf(mt, m[b][cc], old[b][cc]) : mt * m[b][cc];
+    });
+    // position terms of the momentum, through the modes
+    adj_position<R, D, false>(X, dX, Y, dY, Z, dZ, lmv, coef, Dx, Dy, Dz);
     lx[0] = fmaf(mt, Dx, lx[0]);
     lx[1] = fmaf(mt, Dy, lx[1]);
     lx[2] = fmaf(mt, Dz, lx[2]);
 }
 
+// Tiles of at most this many particles are walked in memory order (below).
+constexpr int kAdjList = 3072;
+constexpr int kAdjWords = 128;  // bitmap words: a window of 4096 indices
+
+// The tile's particle indices perm[jb .. je) into `idx` in ascending order:
+// those inside a window of 4096 around the median of three samples ranked by a
+// bitmap, the others behind them in any order (every particle reads and writes
+// only its own entries, so the order changes no result).  The arrays are in
+// the slot order of the step before: ascending indices read and write whole
+// sectors of their 162 coefficient rows where slot order, moved by a rank
+// wherever a particle left or entered a cell, touched them in pieces.
+__device__ __forceinline__ void list_in_memory_order(const uint32_t *__restrict__ perm, uint32_t jb,
+                                                     uint32_t je, uint32_t *idx, uint32_t *bits) {
+    uint32_t *pre = bits + kAdjWords, *far = pre + kAdjWords;
+    const uint32_t n = je - jb;
+    const uint32_t a = perm[jb + n / 4], b = perm[jb + n / 2], c = perm[jb + (n - 1) - n / 4];
+    const uint32_t mid = max(min(a, b), min(max(a, b), c));
+    constexpr uint32_t W = 32 * kAdjWords;
+    const uint32_t base = mid > W / 2 ? (mid - W / 2) & ~31u : 0u;
+    for (int i = threadIdx.x; i < kAdjWords; i += blockDim.x) bits[i] = 0;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint32_t off = perm[jb + i] - base;
+        if (off < W) atomicOr(&bits[off >> 5], 1u << (off & 31u));
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        uint32_t run = 0;
+        for (int w0 = 0; w0 < kAdjWords; w0 += 32) {
+            const uint32_t v = (uint32_t)__popc(bits[w0 + lane]);
+            uint32_t x = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            pre[w0 + lane] = run + x - v;
+            run += __shfl_sync(0xffffffffu, x, 31);
+        }
+        if (lane == 0) *far = run;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint32_t p = perm[jb + i], off = p - base;
+        const uint32_t at = off < W ? pre[off >> 5] + (uint32_t)__popc(bits[off >> 5] &
+                                                                     ((1u << (off & 31u)) - 1u))
+                                    : atomicAdd(far, 1u);
+        if (at < n) idx[at] = p;  // perm names n distinct particles
+    }
+    __syncthreads();
+}
+
 template <int R>
-__global__ void __launch_bounds__(kAdjThreads) k_p2g_adjoint(AdjP2GArgs Q) {
+__global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(AdjP2GArgs Q) {
     extern __shared__ float s_adj[];
+    __shared__ uint32_t s_idx[kAdjList], s_bits[2 * kAdjWords + 1];
     float *tile_m = s_adj, *tile_v = s_adj + kATileFloats;
     const GridGeom &g = Q.g;
     const uint32_t tile = blockIdx.x;
@@ -444,23 +529,31 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adjoint(AdjP2GArgs Q) {
     const int ox = 8 * tx - 1, oy = 8 * ty - 1, oz = 4 * tz - 1;
     stage_tile(g, Q.lm, ox, oy, oz, tile_m);
     stage_tile(g, Q.lmv, ox, oy, oz, tile_v);
-    __syncthreads();
+    const bool listed = je - jb <= (uint32_t)kAdjList;  // CTA-uniform
+    if (listed) list_in_memory_order(Q.perm, jb, je, s_idx, s_bits);
+    else __syncthreads();
+    auto particle = [&](uint32_t j) { return listed ? s_idx[j - jb] : Q.perm[j]; };
     // software pipeline: the next particle's index, position and mass load
-    // while this one is computed
+    // while this one is computed, every component's coefficients one ahead
+    CoeffStage<R> coef(s_adj + 2 * kATileFloats);
+    const int64_t cnt = Q.count;
     uint32_t j = jb + threadIdx.x;
-    uint32_t pn = j < je ? Q.perm[j] : 0u;
+    uint32_t pn = j < je ? particle(j) : 0u;
     float nx = 0.0f, ny = 0.0f, nz = 0.0f, nm = 0.0f;
     if (j < je) {
         nx = Q.x[0][pn];
         ny = Q.x[1][pn];
         nz = Q.x[2][pn];
         nm = Q.mass[pn] + (Q.mass_abs ? Q.mass_abs[pn] : 0.0f);
+        coef.fill(false, Q.coeff + pn, cnt);
     }
+    cp_async_commit();
     for (; j < je; j += kAdjThreads) {
         const uint32_t p = pn;
         const float px = nx, py = ny, pz = nz, mt = nm;
-        if (j + kAdjThreads < je) {
-            pn = Q.perm[j + kAdjThreads];
+        const bool more = j + kAdjThreads < je;
+        if (more) {
+            pn = particle(j + kAdjThreads);
             nx = Q.x[0][pn];
             ny = Q.x[1][pn];
             nz = Q.x[2][pn];
@@ -468,11 +561,19 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adjoint(AdjP2GArgs Q) {
         }
         const ParticleAxes pa = particle_axes(g, px, py, pz, tx, ty, tz);
         float lx[3] = {0.0f, 0.0f, 0.0f};
-        if (pa.ok) {
-            p2g_adj_component<R, 0>(Q, pa, tile_m, tile_v, ox, oy, oz, p, mt, lx);
-            p2g_adj_component<R, 1>(Q, pa, tile_m, tile_v, ox, oy, oz, p, mt, lx);
-            p2g_adj_component<R, 2>(Q, pa, tile_m, tile_v, ox, oy, oz, p, mt, lx);
-        } else {
+        auto component = [&](auto axis) {
+            constexpr int A = decltype(axis)::value;
+            if (A < 2) coef.fill(true, Q.coeff + (int64_t)(A + 1) * R * cnt + p, cnt);
+            else if (more) coef.fill(true, Q.coeff + pn, cnt);
+            cp_async_commit();
+            cp_async_wait<1>();
+            if (pa.ok) p2g_adj_component<R, A>(Q, pa, tile_m, tile_v, ox, oy, oz, p, mt, coef, lx);
+            coef.next();
+        };
+        component(std::integral_constant<int, 0>{});
+        component(std::integral_constant<int, 1>{});
+        component(std::integral_constant<int, 2>{});
+        if (!pa.ok) {
             atomicOr(Q.status, kFlagOutOfDomain);
             for (int a = 0; a < 3; ++a)
                 for (int r = 0; r < R; ++r) {
@@ -492,8 +593,26 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adjoint(AdjP2GArgs Q) {
 }
 
 // ---------------------------------------------------------------- drivers
-size_t adjoint_scratch_bytes(int64_t count, int R) {
-    return (size_t)count * 3 * R * sizeof(float) + 512;
+size_t adjoint_scratch_bytes(int64_t count) {
+    return (size_t)count * 3 * sizeof(float) + 512;
+}
+
+template <int R>
+static cudaError_t launch_g2p_adjoint(const AdjG2PArgs &G, int64_t tiles, cudaStream_t s) {
+    constexpr int smem = stage_bytes<R>();
+    const cudaError_t e = cudaFuncSetAttribute(k_g2p_adjoint<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_g2p_adjoint<R><<<(int)tiles, kAdjThreads, smem, s>>>(G);
+    return cudaGetLastError();
+}
+
+template <int R>
+static cudaError_t launch_p2g_adjoint(const AdjP2GArgs &Q, int64_t tiles, cudaStream_t s) {
+    constexpr int smem = stage_bytes<R>() + 2 * kATileFloats * (int)sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(k_p2g_adjoint<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_p2g_adjoint<R><<<(int)tiles, kAdjThreads, smem, s>>>(Q);
+    return cudaGetLastError();
 }
 
 cudaError_t adjoint_g2p(const GridGeom &g, int64_t num_keys, int R, float dx,
@@ -511,7 +630,7 @@ cudaError_t adjoint_g2p(const GridGeom &g, int64_t num_keys, int R, float dx,
             }
         return cudaSuccess;
     }
-    float *mu = ws.take<float>((size_t)in->count * 3 * R);
+    float *mu0 = ws.take<float>((size_t)in->count * 3);
     P2GArgs P{};
     P.scratch = ws.take<float>((size_t)tiles * kTileFloats);
     P.tile_live = ws.take<uint8_t>((size_t)tiles);
@@ -531,14 +650,14 @@ cudaError_t adjoint_g2p(const GridGeom &g, int64_t num_keys, int R, float dx,
     G.bar_c = static_cast<const float *>(bar_out->coeff);
     G.perm = in->perm;
     G.cell_start = in->cell_start;
-    G.mu = mu;
+    G.mu0 = mu0;
     G.status = status;
     G.accumulate = accumulate;
     cudaError_t e = cudaErrorInvalidValue;
-    if (R == 1) { k_g2p_adjoint<1><<<(int)tiles, kAdjThreads, 0, s>>>(G); e = cudaGetLastError(); }
-    if (R == 4) { k_g2p_adjoint<4><<<(int)tiles, kAdjThreads, 0, s>>>(G); e = cudaGetLastError(); }
-    if (R == 8) { k_g2p_adjoint<8><<<(int)tiles, kAdjThreads, 0, s>>>(G); e = cudaGetLastError(); }
-    if (R == 27) { k_g2p_adjoint<27><<<(int)tiles, kAdjThreads, 0, s>>>(G); e = cudaGetLastError(); }
+    if (R == 1) e = launch_g2p_adjoint<1>(G, tiles, s);
+    if (R == 4) e = launch_g2p_adjoint<4>(G, tiles, s);
+    if (R == 8) e = launch_g2p_adjoint<8>(G, tiles, s);
+    if (R == 27) e = launch_g2p_adjoint<27>(G, tiles, s);
     if (e != cudaSuccess) return e;
 
     P.g = g;
@@ -551,7 +670,8 @@ cudaError_t adjoint_g2p(const GridGeom &g, int64_t num_keys, int R, float dx,
     P.status = status;
     P.nblocks = (uint32_t)(num_keys / 32);
     P.s1 = P.s2 = 1.0f;  // the scatter's fit rows carry their own 1/dx powers
-    P.mu = mu;
+    P.mu = static_cast<const float *>(bar_out->coeff);
+    P.mu0 = mu0;
     P.inv_dx = 1.0f / dx;
     P.inv_dx2 = 1.0f / (dx * dx);
     return p2g_adjoint_scatter(P, bar_grid->vel, accumulate, R, s);
@@ -583,17 +703,10 @@ cudaError_t adjoint_p2g(const GridGeom &g, int64_t num_keys, int R, float dx,
     Q.status = status;
     Q.accumulate = accumulate;
     const int64_t tiles = num_keys / 256;
-    const int smem = 2 * kATileFloats * (int)sizeof(float);
-#define POLYPIC_ADJ_CASE(RR)                                                        \
-    if (R == RR) {                                                                  \
-        k_p2g_adjoint<RR><<<(int)tiles, kAdjThreads, smem, s>>>(Q);                \
-        return cudaGetLastError();                                                  \
-    }
-    POLYPIC_ADJ_CASE(1)
-    POLYPIC_ADJ_CASE(4)
-    POLYPIC_ADJ_CASE(8)
-    POLYPIC_ADJ_CASE(27)
-#undef POLYPIC_ADJ_CASE
+    if (R == 1) return launch_p2g_adjoint<1>(Q, tiles, s);
+    if (R == 4) return launch_p2g_adjoint<4>(Q, tiles, s);
+    if (R == 8) return launch_p2g_adjoint<8>(Q, tiles, s);
+    if (R == 27) return launch_p2g_adjoint<27>(Q, tiles, s);
     return cudaErrorInvalidValue;
 }
 

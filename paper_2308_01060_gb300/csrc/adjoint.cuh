@@ -13,7 +13,8 @@ struct AdjG2PArgs {
     const float *bar_x[3];        // dL/dx' (slot order)
     const float *bar_c;           // dL/dc' [3][R][count] (slot order)
     const uint32_t *perm, *cell_start;
-    float *mu;                    // out: effective coefficient adjoint (slot order)
+    float *mu0;                   // out: [3][count] effective adjoint of the constant modes
+                                  // (slot order); the other modes' is bar_c itself
     float *out_x[3];              // out: dL/dx (storage order)
     uint32_t *status;
     bool accumulate;
@@ -34,7 +35,7 @@ struct AdjP2GArgs {
     bool accumulate;
 };
 
-size_t adjoint_scratch_bytes(int64_t count, int R);
+size_t adjoint_scratch_bytes(int64_t count);
 
 cudaError_t adjoint_g2p(const GridGeom &g, int64_t num_keys, int R, float dx,
                         const polypic_grid *grid, const polypic_particles *in, float dt,

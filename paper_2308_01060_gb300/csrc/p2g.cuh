@@ -46,8 +46,9 @@ struct P2GArgs {
     // Eq 12's affine map (4 modes, FP32): M = (I + map_dt C_p)^-1
     bool affine;
     float map_dt;
-    // adjoint scatter only: mu [3][R][count] in slot order, 1/dx, 1/dx^2
-    const float *mu;
+    // adjoint scatter only: the coefficient adjoint mu [3][R][count] in slot order,
+    // its constant modes in mu0 [3][count] instead; 1/dx, 1/dx^2
+    const float *mu, *mu0;
     float inv_dx, inv_dx2;
 };
 

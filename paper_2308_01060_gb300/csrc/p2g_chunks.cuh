@@ -335,7 +335,9 @@ __device__ __forceinline__ void p2g_item(const P2GArgs &P, uint32_t tile, int g,
         // adjoint scatter: coefficients mu in slot order
         const uint32_t *c = rows + (ADJ ? slot : p);
 #pragma unroll
-        for (int r = 0; r < H; ++r) cp_async4(st + r * 32, c + (uint64_t)cnt * (uint32_t)r);
+        for (int r = ADJ ? 1 : 0; r < H; ++r)
+            cp_async4(st + r * 32, c + (uint64_t)cnt * (uint32_t)r);
+        if constexpr (ADJ) cp_async4(st, P.mu0 + (uint64_t)cnt * (uint32_t)a + slot);
         if constexpr (AFF) {
             const float *cf = reinterpret_cast<const float *>(P.coeff) + p;
 #pragma unroll

@@ -3,6 +3,7 @@
 // particle, the sum-factorised accumulation into a lane's padded 4 x 3 x 3
 // footprint, and the slot of a lane's particle in a round.
 #pragma once
+#include "cp_async.cuh"
 #include "p2g.cuh"
 
 namespace polypic {
@@ -57,17 +58,6 @@ template <int R, bool AFF = false, int FMT = POLYPIC_COEFF_F32> struct Stage {
     static constexpr int NV = kL + (AFF ? 6 : 0);
 };
 
-__device__ __forceinline__ void cp_async4(float *dst, const void *src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
 template <int R, int FMT, int A, bool ADJ, bool AFF = false>
 __device__ __forceinline__ void stage_particle(const P2GArgs &P, uint32_t p, uint32_t slot,
                                                float *st, int lane) {
@@ -76,11 +66,12 @@ __device__ __forceinline__ void stage_particle(const P2GArgs &P, uint32_t p, uin
     cp_async4(st + S::kY * 32 + lane, P.y + p);
     cp_async4(st + S::kZ * 32 + lane, P.z + p);
     if constexpr (ADJ) {
-        // adjoint scatter: unit weight, coefficients mu (slot order) from scratch
+        // adjoint scatter: unit weight, coefficients mu (slot order)
         st[S::kM * 32 + lane] = 1.0f;
-        const float *c = P.mu + (int64_t)A * R * P.count + slot;
+        cp_async4(st + S::kC * 32 + lane, P.mu0 + (int64_t)A * P.count + slot);
+        const float *c = P.mu + ((int64_t)A * R + 1) * P.count + slot;
 #pragma unroll
-        for (int r = 0; r < R; ++r, c += P.count) cp_async4(st + (S::kC + r) * 32 + lane, c);
+        for (int r = 1; r < R; ++r, c += P.count) cp_async4(st + (S::kC + r) * 32 + lane, c);
         return;
     }
     cp_async4(st + S::kM * 32 + lane, P.mass + p);
