@@ -187,11 +187,11 @@ def algorithmic_bytes(R: int, fmt: str):
 
 def launches_per_step() -> int:
     """Kernels of ours per polypic_step (one phase, no projection): keys with
-    arrival ranks, the 3-kernel count scan, the scatter, the per-cell order,
+    arrival ranks, the 2-kernel count scan, the scatter, the per-cell order,
     the crowded-cell pass (exits at once when no cell holds more than 64
     particles), P2G tiles + the tile reduction with the grid update fused in,
     G2P."""
-    return 1 + 3 + 1 + 1 + 1 + 2 + 1
+    return 1 + 2 + 1 + 1 + 1 + 2 + 1
 
 
 def make_state(pp, ctx, scene, device):

@@ -39,10 +39,14 @@ __global__ void __launch_bounds__(256) k_keys(int64_t n, const float *__restrict
                                               uint32_t *__restrict__ rank,
                                               uint32_t *__restrict__ counts,
                                               uint32_t *__restrict__ num_crowded,
+                                              uint32_t *__restrict__ arrived,
                                               uint32_t *__restrict__ status) {
     const int lane = threadIdx.x & 31;
     const int64_t base = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * (32 * kKeyRuns) + lane;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *num_crowded = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *num_crowded = 0;
+        *arrived = 0;
+    }
     uint32_t k[kKeyRuns];
     bool bad = false;
 #pragma unroll
@@ -118,37 +122,105 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *s
     return r;
 }
 
+// Totals of kScanTile chunks; the CTA that arrives last (no CTA waits for
+// another) turns them into their exclusive prefix, nb <= kScanThreads * 256.
+// *arrived is 0 before and after.
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *__restrict__ in,
-                                                              int64_t L,
-                                                              uint32_t *__restrict__ sums) {
+                                                              int64_t L, uint32_t *sums,
+                                                              uint32_t *arrived) {
     __shared__ uint32_t s_warp[33];
+    __shared__ bool last;
     int64_t base = (int64_t)blockIdx.x * kScanTile;
     uint32_t acc = 0;
-    for (int i = threadIdx.x; i < kScanTile; i += kScanThreads) {
-        int64_t idx = base + i;
+#pragma unroll
+    for (int i = 0; i < kScanTile / kScanThreads; ++i) {
+        int64_t idx = base + i * kScanThreads + threadIdx.x;
         if (idx < L) acc += in[idx];
     }
     uint32_t total;
     block_exclusive_scan(acc, s_warp, &total);
-    if (threadIdx.x == 0) sums[blockIdx.x] = total;
-}
-
-// Single-CTA exclusive scan of nb block sums (nb <= kScanThreads * 256).
-__global__ void __launch_bounds__(kScanThreads) k_scan_top(uint32_t *__restrict__ sums, int nb) {
-    __shared__ uint32_t s_warp[33];
-    int per = (nb + kScanThreads - 1) / kScanThreads;
-    int beg = threadIdx.x * per;
-    uint32_t acc = 0;
+    if (threadIdx.x == 0) {
+        sums[blockIdx.x] = total;
+        __threadfence();
+        last = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1;  // wraps to 0
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    volatile uint32_t *v = sums;
+    const int nb = (int)gridDim.x;
+    const int per = (nb + kScanThreads - 1) / kScanThreads;
+    const int beg = threadIdx.x * per;
+    acc = 0;
     for (int i = 0; i < per; ++i)
-        if (beg + i < nb) acc += sums[beg + i];
-    uint32_t total;
+        if (beg + i < nb) acc += v[beg + i];
     uint32_t run = block_exclusive_scan(acc, s_warp, &total);
     for (int i = 0; i < per; ++i)
         if (beg + i < nb) {
-            uint32_t v = sums[beg + i];
-            sums[beg + i] = run;
-            run += v;
+            const uint32_t x = v[beg + i];
+            v[beg + i] = run;
+            run += x;
         }
+}
+
+// Exclusive scan of at most kScanOne counts in one CTA, kScanPart at a time:
+// every warp takes 1/32 of a part, its loads all in flight at once, then the
+// warps' totals.  K is a multiple of 256; out[K] gets the total.
+constexpr int kScanOne = 65536, kScanPart = 32768;
+__global__ void __launch_bounds__(1024) k_scan_one(const uint32_t *in, uint32_t *out, int K) {
+    __shared__ uint32_t s_warp[33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int kIts = kScanPart / 32 / 128;  // 128 counts per warp and step
+    uint32_t carry = 0;
+    for (int p0 = 0; p0 < K; p0 += kScanPart) {
+        const int end = min(K, p0 + kScanPart);
+        const int per = ((end - p0) / 128 + 31) / 32;  // steps of a warp
+        const int base = p0 + w * per * 128 + lane * 4;
+        uint4 v[kIts];
+#pragma unroll
+        for (int i = 0; i < kIts; ++i) {
+            v[i] = make_uint4(0, 0, 0, 0);
+            if (i < per && base + i * 128 < end)
+                v[i] = *reinterpret_cast<const uint4 *>(in + base + i * 128);
+        }
+        uint32_t run = 0;  // before the lane's first count of the step
+#pragma unroll
+        for (int i = 0; i < kIts; ++i) {
+            const uint32_t a = v[i].x, b = a + v[i].y, c = b + v[i].z, d = c + v[i].w;
+            uint32_t incl = d;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const uint32_t ex = run + incl - d;
+            v[i] = make_uint4(ex, ex + a, ex + b, ex + c);
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) s_warp[w] = run;
+        __syncthreads();
+        if (w == 0) {
+            const uint32_t t = s_warp[lane];
+            uint32_t incl = t;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            s_warp[lane] = incl - t;
+            if (lane == 31) s_warp[32] = incl;
+        }
+        __syncthreads();
+        const uint32_t before = carry + s_warp[w];
+#pragma unroll
+        for (int i = 0; i < kIts; ++i)
+            if (i < per && base + i * 128 < end)
+                *reinterpret_cast<uint4 *>(out + base + i * 128) =
+                    make_uint4(v[i].x + before, v[i].y + before, v[i].z + before, v[i].w + before);
+        carry += s_warp[32];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[K] = carry;
 }
 
 // Exclusive scan of one kScanTile chunk plus its block offset, in place
@@ -188,14 +260,20 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t *in, 
 
 size_t scan_scratch_words(int64_t L) { return (size_t)((L + kScanTile - 1) / kScanTile) + 1; }
 
-cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, int64_t L, uint32_t *scratch,
-                           cudaStream_t s) {
-    if (L <= 0) return cudaSuccess;
-    int nb = (int)((L + kScanTile - 1) / kScanTile);
+// Exclusive prefix of the key counts cs[0 .. K), in place, cs[K] their total
+// (K is a multiple of 256).  scratch: scan_scratch_words(K + 1) words, the last
+// of them 0 on entry.
+static cudaError_t scan_counts(uint32_t *cs, int64_t K, uint32_t *scratch, cudaStream_t s) {
+    // one CTA reads and writes 16 bytes at a time
+    if (K <= kScanOne && ((uintptr_t)cs & 15u) == 0) {
+        k_scan_one<<<1, 1024, 0, s>>>(cs, cs, (int)K);
+        return cudaGetLastError();
+    }
+    const int64_t L = K + 1;
+    const int nb = (int)((L + kScanTile - 1) / kScanTile);
     if (nb > kScanThreads * 256) return cudaErrorInvalidValue;
-    k_scan_reduce<<<nb, kScanThreads, 0, s>>>(in, L, scratch);
-    k_scan_top<<<1, kScanThreads, 0, s>>>(scratch, nb);
-    k_scan_down<<<nb, kScanThreads, 0, s>>>(in, out, L, scratch);
+    k_scan_reduce<<<nb, kScanThreads, 0, s>>>(cs, L, scratch, scratch + nb);
+    k_scan_down<<<nb, kScanThreads, 0, s>>>(cs, cs, L, scratch);
     return cudaGetLastError();
 }
 
@@ -384,7 +462,7 @@ bool take_sort_scratch(Workspace &ws, int64_t count, int64_t num_keys, SortScrat
 cudaError_t finish_order(int64_t num_keys, int64_t count, const uint32_t *key,
                          uint32_t *cell_start, uint32_t *perm, const SortScratch &S,
                          cudaStream_t s) {
-    cudaError_t e = exclusive_scan(cell_start, cell_start, num_keys + 1, S.cscan, s);
+    cudaError_t e = scan_counts(cell_start, num_keys, S.cscan, s);
     if (e != cudaSuccess) return e;
     const int pblocks = (int)((count + 255) / 256);
     k_scatter<<<pblocks, 256, 0, s>>>(count, key, S.rank, cell_start, S.arrival);
@@ -409,7 +487,8 @@ cudaError_t sort_particles(const GridGeom &g, int64_t num_keys, int64_t count, c
     if (!take_sort_scratch(ws, count, num_keys, S)) return cudaErrorInvalidValue;
     if (!key) key = S.key;
     k_keys<<<(int)((count + 256 * kKeyRuns - 1) / (256 * kKeyRuns)), 256, 0, s>>>(
-        count, x, y, z, g, key, S.rank, cell_start, S.num_crowded, status);
+        count, x, y, z, g, key, S.rank, cell_start, S.num_crowded,
+        S.cscan + scan_scratch_words(num_keys + 1) - 1, status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return finish_order(num_keys, count, key, cell_start, perm, S, s);
 }

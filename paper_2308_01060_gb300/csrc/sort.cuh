@@ -10,12 +10,8 @@ constexpr int kScanTile = 4096;
 // selection (quadratic in the population); larger ones by a CTA radix sort.
 constexpr int kSelectMax = 64;
 
+// Words of the count scan's scratch for L counts.
 size_t scan_scratch_words(int64_t L);
-
-// Exclusive prefix sum of L uint32 (in may equal out); scratch holds
-// scan_scratch_words(L) words.
-cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, int64_t L, uint32_t *scratch,
-                           cudaStream_t s);
 
 // Scratch of one sort, carved from the caller's workspace.
 struct SortScratch {
