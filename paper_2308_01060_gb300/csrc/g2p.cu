@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kG2PThreads) k_g2p_tiles(G2PArgs A) {
 
     using T = typename Codec<FMT>::T;
     T *ocoeff = reinterpret_cast<T *>(A.ocoeff);
-    const int64_t cnt = A.count;
+    const uint32_t cnt = (uint32_t)A.count;  // rows are count < 2^31 words apart
     // FP32 output is physical (c = c dx^L / dx^L); the 16-bit codes take c dx^L
     const float inv1 = FMT == POLYPIC_COEFF_F32 ? A.inv_dxpow[1] : 1.0f;
     const float inv2 = FMT == POLYPIC_COEFF_F32 ? A.inv_dxpow[2] : 1.0f;
@@ -120,7 +120,8 @@ __global__ void __launch_bounds__(kG2PThreads) k_g2p_tiles(G2PArgs A) {
                 float C[R];
                 fit(acomp, C);
 #pragma unroll
-                for (int r = 0; r < R; ++r, out += cnt) *out = C[r];
+                for (int r = 0; r < R; ++r)
+                    out[(uint64_t)cnt * (uint32_t)(decltype(acomp)::value * R + r)] = C[r];
                 vel[decltype(acomp)::value] = C[0];
             };
             fit_store(std::integral_constant<int, 0>{});
@@ -143,11 +144,11 @@ __global__ void __launch_bounds__(kG2PThreads) k_g2p_tiles(G2PArgs A) {
 #pragma unroll
             for (int a = 0; a < 3; ++a)
 #pragma unroll
-                for (int k = 0; k < H; ++k, ow += cnt) {
+                for (int k = 0; k < H; ++k) {
                     const uint32_t lo = Codec<FMT>::bits(Codec<FMT>::encode(Chat[a][2 * k] * inv));
                     const uint32_t hi = 2 * k + 1 < R
                         ? Codec<FMT>::bits(Codec<FMT>::encode(Chat[a][2 * k + 1] * inv)) : 0u;
-                    *ow = lo | (hi << 16);
+                    ow[(uint64_t)cnt * (uint32_t)(a * H + k)] = lo | (hi << 16);
                 }
             A.oscale[j] = s;
 #pragma unroll

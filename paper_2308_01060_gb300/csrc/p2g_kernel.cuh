@@ -58,48 +58,45 @@ template <int R, bool AFF = false, int FMT = POLYPIC_COEFF_F32> struct Stage {
     static constexpr int NV = kL + (AFF ? 6 : 0);
 };
 
-template <int R, int FMT, int A, bool ADJ, bool AFF = false>
-__device__ __forceinline__ void stage_particle(const P2GArgs &P, uint32_t p, uint32_t slot,
+// Face grid A is a run-time value here: one copy of the loads serves the three
+// passes.  Rows are P.count < 2^31 words apart.
+template <int R, int FMT, bool ADJ, bool AFF = false>
+__device__ __forceinline__ void stage_particle(const P2GArgs &P, int A, uint32_t p, uint32_t slot,
                                                float *st, int lane) {
     using S = Stage<R, AFF, FMT>;
-    cp_async4(st + S::kX * 32 + lane, P.x + p);
-    cp_async4(st + S::kY * 32 + lane, P.y + p);
-    cp_async4(st + S::kZ * 32 + lane, P.z + p);
+    const uint32_t cnt = (uint32_t)P.count;
+    st += lane;
+    cp_async4(st + S::kX * 32, P.x + p);
+    cp_async4(st + S::kY * 32, P.y + p);
+    cp_async4(st + S::kZ * 32, P.z + p);
     if constexpr (ADJ) {
         // adjoint scatter: unit weight, coefficients mu (slot order)
-        st[S::kM * 32 + lane] = 1.0f;
-        cp_async4(st + S::kC * 32 + lane, P.mu0 + (int64_t)A * P.count + slot);
-        const float *c = P.mu + ((int64_t)A * R + 1) * P.count + slot;
+        st[S::kM * 32] = 1.0f;
+        cp_async4(st + S::kC * 32, P.mu0 + (uint64_t)cnt * (uint32_t)A + slot);
+        const float *c = P.mu + (uint64_t)cnt * (uint32_t)(A * R) + slot;
 #pragma unroll
-        for (int r = 1; r < R; ++r, c += P.count) cp_async4(st + (S::kC + r) * 32 + lane, c);
+        for (int r = 1; r < R; ++r)
+            cp_async4(st + (S::kC + r) * 32, c + (uint64_t)cnt * (uint32_t)r);
         return;
     }
-    cp_async4(st + S::kM * 32 + lane, P.mass + p);
-    if (P.mass_abs) cp_async4(st + S::kMabs * 32 + lane, P.mass_abs + p);
-    reinterpret_cast<uint32_t *>(st)[S::kIdx * 32 + lane] = p;
-    if constexpr (FMT == POLYPIC_COEFF_F32) {
-        // row r of component A starts (A R + r) * count floats in
-        const float *c = reinterpret_cast<const float *>(P.coeff) + (int64_t)A * R * P.count + p;
+    cp_async4(st + S::kM * 32, P.mass + p);
+    if (P.mass_abs) cp_async4(st + S::kMabs * 32, P.mass_abs + p);
+    if constexpr (FMT != POLYPIC_COEFF_F32) cp_async4(st + S::kScale * 32, P.scale + p);
+    // FP32: row (A, r) holds mode r; 16-bit codes: word (A, k) modes 2k and 2k + 1
+    constexpr int H = coeff_words(R, FMT);
+    const uint32_t *c = reinterpret_cast<const uint32_t *>(P.coeff) + (uint64_t)cnt * (uint32_t)(A * H) + p;
 #pragma unroll
-        for (int r = 0; r < R; ++r, c += P.count) cp_async4(st + (S::kC + r) * 32 + lane, c);
-        if constexpr (AFF) {
-            const float *cf = reinterpret_cast<const float *>(P.coeff) + p;
+    for (int r = 0; r < H; ++r) cp_async4(st + (S::kC + r) * 32, c + (uint64_t)cnt * (uint32_t)r);
+    if constexpr (AFF) {
+        const float *cf = reinterpret_cast<const float *>(P.coeff) + p;
 #pragma unroll
-            for (int o = 0; o < 2; ++o) {
-                const int a2 = o < A ? o : o + 1;  // the other two components, ascending
+        for (int o = 0; o < 2; ++o) {
+            const int a2 = o < A ? o : o + 1;  // the other two components, ascending
+            const float *co = cf + (uint64_t)cnt * (uint32_t)(a2 * R);
 #pragma unroll
-                for (int b = 0; b < 3; ++b)
-                    cp_async4(st + (S::kL + 3 * o + b) * 32 + lane,
-                              cf + ((int64_t)a2 * R + 1 + b) * P.count);
-            }
+            for (int b = 0; b < 3; ++b)
+                cp_async4(st + (S::kL + 3 * o + b) * 32, co + (uint64_t)cnt * (uint32_t)(1 + b));
         }
-    } else {
-        // 16-bit codes: word (A H + k, p), H = (R + 1) / 2, holds modes 2k and 2k + 1
-        cp_async4(st + S::kScale * 32 + lane, P.scale + p);
-        constexpr int H = coeff_words(R, FMT);
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(P.coeff) + (int64_t)A * H * P.count + p;
-#pragma unroll
-        for (int k = 0; k < H; ++k, w += P.count) cp_async4(st + (S::kC + k) * 32 + lane, w);
     }
 }
 

@@ -39,26 +39,32 @@ static_assert(p2g_smem_bytes<8, true>() <= 227 * 1024,
 struct Pipe {
     int ia;
     uint32_t ir, sn, pn;
+    uint32_t before;  // slots of the block before round ir
     int ring;  // stage holding the next round to consume
+
+    // Slot of the lane's particle in round ir (every lane must call it); the
+    // rounds come in order, so the slots before one are a running sum.
+    __device__ __forceinline__ void locate(const uint32_t *perm, uint32_t bs, uint32_t n_c,
+                                           unsigned lt) {
+        const unsigned mask = __ballot_sync(0xffffffffu, n_c > ir);
+        sn = bs + before + __popc(mask & lt);
+        before += __popc(mask);
+        pn = n_c > ir ? perm[sn] : 0u;
+    }
 };
 
 template <int R, int FMT, bool ADJ, bool AFF>
 __device__ __forceinline__ void pipe_issue(const P2GArgs &P, Pipe &q, uint32_t bs, uint32_t n_c,
                                            uint32_t maxn, unsigned lt, float *st, int lane) {
-    if (q.ia < 3 && n_c > q.ir) {  // q.ia is warp-uniform
-        if (q.ia == 0) stage_particle<R, FMT, 0, ADJ, AFF>(P, q.pn, q.sn, st, lane);
-        else if (q.ia == 1) stage_particle<R, FMT, 1, ADJ, AFF>(P, q.pn, q.sn, st, lane);
-        else stage_particle<R, FMT, 2, ADJ, AFF>(P, q.pn, q.sn, st, lane);
-    }
+    if (q.ia < 3 && n_c > q.ir)  // q.ia is warp-uniform
+        stage_particle<R, FMT, ADJ, AFF>(P, q.ia, q.pn, q.sn, st, lane);
     cp_async_commit();
     if (q.ia < 3 && ++q.ir == maxn) {
         q.ir = 0;
+        q.before = 0;
         ++q.ia;
     }
-    if (q.ia < 3) {
-        q.sn = round_slot(bs, n_c, q.ir, lt);
-        q.pn = n_c > q.ir ? P.perm[q.sn] : 0u;
-    }
+    if (q.ia < 3) q.locate(P.perm, bs, n_c, lt);
 }
 
 template <int R, int FMT, int A, bool ADJ, bool AFF>
@@ -66,8 +72,10 @@ __device__ __forceinline__ void p2g_pass(const P2GArgs &P, Pipe &q, uint32_t bs,
                                          uint32_t maxn, int ci, int cj, int ck, int gi, int gj,
                                          int gk, int lane, float *reg, float *stage, bool &bad) {
     using S = Stage<R, AFF, FMT>;
-    const bool interior = gi >= 1 && gi <= P.g.n[0] - 2 && gj >= 1 && gj <= P.g.n[1] - 2 &&
-                          gk >= 1 && gk <= P.g.n[2] - 2;
+    // being in a cell of 1 .. n - 2 on every axis is the valid region 1 <= v < n - 1
+    const bool valid = gi >= 1 && gi <= P.g.n[0] - 2 && gj >= 1 && gj <= P.g.n[1] - 2 &&
+                       gk >= 1 && gk <= P.g.n[2] - 2;
+    const float fi = (float)gi, fj = (float)gj, fk = (float)gk;
     Foot F;
     F.zero();
     const unsigned lt = (1u << lane) - 1u;
@@ -81,10 +89,7 @@ __device__ __forceinline__ void p2g_pass(const P2GArgs &P, Pipe &q, uint32_t bs,
             if (!ADJ && P.mass_abs) mt += st[S::kMabs * 32 + lane];
             const float v0 = cell_coord(px, P.g.inv_dx), v1 = cell_coord(py, P.g.inv_dx),
                         v2 = cell_coord(pz, P.g.inv_dx);
-            // in an interior cell, being in the cell implies the valid region
-            const bool ok = (interior || (coord_valid(v0, P.g.n[0]) && coord_valid(v1, P.g.n[1]) &&
-                                          coord_valid(v2, P.g.n[2]))) &&
-                            (int)floorf(v0) == gi && (int)floorf(v1) == gj && (int)floorf(v2) == gk;
+            const bool ok = valid && floorf(v0) == fi && floorf(v1) == fj && floorf(v2) == fk;
             if (ok) {
                 const float vu = A == 0 ? v0 : (A == 1 ? v1 : v2);
                 const float vv = A == 0 ? v1 : v0;
@@ -137,8 +142,8 @@ __device__ __forceinline__ void p2g_block(const P2GArgs &P, uint32_t bs, uint32_
     q.ia = 0;
     q.ir = 0;
     q.ring = 0;
-    q.sn = round_slot(bs, n_c, 0, lt);
-    q.pn = n_c > 0 ? P.perm[q.sn] : 0u;
+    q.before = 0;
+    q.locate(P.perm, bs, n_c, lt);
 #pragma unroll
     for (int k = 0; k < kStages; ++k)
         pipe_issue<R, FMT, ADJ, AFF>(P, q, bs, n_c, maxn, lt, stage + k * Stage<R, AFF, FMT>::NV * 32,
