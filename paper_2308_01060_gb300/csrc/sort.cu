@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(256) k_scatter(int64_t n, const uint32_t *__re
 // n^2 over its cells / 32 loads, not the fullest cell's n^2.  Cells holding
 // more than kSelectMax particles are listed for k_crowded_cells instead and
 // their slots are left to it.
+constexpr int kOrderStage = 512;
 __global__ void __launch_bounds__(256) k_cell_order(const uint32_t *__restrict__ in,
                                                     const uint32_t *__restrict__ cs,
                                                     uint32_t *__restrict__ out, uint32_t nblocks,
@@ -308,6 +309,7 @@ __global__ void __launch_bounds__(256) k_cell_order(const uint32_t *__restrict__
                                                     uint32_t *__restrict__ num_crowded) {
     __shared__ uint32_t s_tab[8][2][kSelectMax];
     __shared__ uint32_t s_start[8][33];
+    __shared__ uint32_t s_in[8][kOrderStage];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t b = blockIdx.x * 8 + w;
     if (b >= nblocks) return;  // warp-uniform
@@ -328,6 +330,12 @@ __global__ void __launch_bounds__(256) k_cell_order(const uint32_t *__restrict__
     }
     s_start[w][lane] = s0;
     if (lane == 0) s_start[w][32] = end;
+    // the block's arrival list, which every particle of a cell reads again (from
+    // global memory: 35.5 instead of 32.7 us for 3.8 million particles, 10.4
+    // instead of 7.6 for 119 thousand)
+    const bool staged = end - base <= (uint32_t)kOrderStage;  // warp-uniform
+    if (staged)
+        for (uint32_t i = lane; i < end - base; i += 32) s_in[w][i] = in[base + i];
     __syncwarp();
     for (uint32_t i = base + lane; i < end; i += 32) {
         // the cell of arrival slot i: the last lane whose start is <= i
@@ -337,9 +345,16 @@ __global__ void __launch_bounds__(256) k_cell_order(const uint32_t *__restrict__
             if (s_start[w][c + step] <= i) c += step;
         const uint32_t cs0 = s_start[w][c], cn = s_start[w][c + 1] - cs0;
         if (cn > (uint32_t)kSelectMax) continue;  // a crowded cell
-        const uint32_t e = __ldg(in + i);
-        uint32_t rank = 0;
-        for (uint32_t j = 0; j < cn; ++j) rank += __ldg(in + cs0 + j) < e ? 1u : 0u;
+        uint32_t e, rank = 0;
+        if (staged) {
+            const uint32_t *cell = &s_in[w][cs0 - base];
+            e = s_in[w][i - base];
+#pragma unroll 4
+            for (uint32_t j = 0; j < cn; ++j) rank += cell[j] < e ? 1u : 0u;
+        } else {
+            e = __ldg(in + i);
+            for (uint32_t j = 0; j < cn; ++j) rank += __ldg(in + cs0 + j) < e ? 1u : 0u;
+        }
         out[base + tabS[rank] + __popc(tabM[rank] & ((1u << c) - 1u))] = e;
     }
 }
