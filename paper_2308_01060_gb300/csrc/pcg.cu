@@ -27,9 +27,10 @@
 // run one kernel per pass over a list of their fluid cells, in ascending order;
 // all smaller levels run in one CTA from shared memory.  The working set stays in L2
 // (60 MB at 128^3); a pass is bound by its loads' latency and by launching.
-// 128^3 with 476 thousand fluid cells, 24 iterations: 4.68 ms before, with a
-// thread per cell of the box on every level, 23 launches per iteration and the
-// coarsest level's operator read from memory on each of its 32 sweeps.
+// The grid update of 128^3 with 476 thousand fluid cells, 24 iterations, takes
+// 2.23 ms; 4.68 ms before, with a thread per cell of the box on every level,
+// 23 launches per iteration and the coarsest level's operator read from memory
+// on each of its 32 sweeps.
 #include <algorithm>
 #include <cmath>
 #include <new>
@@ -435,7 +436,8 @@ struct MgSmall {
     MgLevel L[kMgMaxLevels];
 };
 
-// Words of shared memory per cell of a small level: the operator and three vectors.
+// Words of shared memory per cell of a small level: the operator and three
+// vectors (the first of several levels: the vectors alone).
 constexpr int kMgWords = 8;
 
 struct SmallLevel {
@@ -456,12 +458,53 @@ struct SmallLevel {
     }
 };
 
-// The rest of the cycle below the large levels, in one CTA: operators and
-// vectors of all small levels in shared memory (16^3 cells and below: 150 KB),
-// the passes separated by the CTA's barrier; the coarsest level keeps each
-// cell's operator in registers for its sweeps.  Cells that are not fluid have
-// wd = b = 0 and only zero couplings: they are computed like the others, and
-// stay finite.  (Launched one by one, the three smallest levels of 128^3 took
+// A thread's cells tid + 1024 k of the first small level, their operator in
+// registers (a neighbour outside is the cell itself, times 0): its passes then
+// read shared memory for the vector alone, 8 words a cell instead of 15, and
+// all the operator's loads are in flight at once: 18.1 -> 16.7 us a cycle with
+// 4,032 and 504 cells.
+constexpr int kMgOwn = (int)((kMgSmall + kMgSmallThreads - 1) / kMgSmallThreads);
+struct OwnCells {
+    float diag[kMgOwn], wd[kMgOwn], o[kMgOwn][6];
+    __device__ __forceinline__ void load(const MgLevel &G, int tid) {
+        const int sy = G.n[0], sz = G.n[0] * G.n[1], cells = (int)G.cells;
+#pragma unroll
+        for (int q = 0; q < kMgOwn; ++q) {
+            const int c = tid + q * kMgSmallThreads;
+            const bool in = c < cells;
+            diag[q] = in ? G.diag[c] : 0.0f;
+            wd[q] = in ? G.wd[c] : 0.0f;
+            o[q][0] = in && c >= 1 ? G.ox[c - 1] : 0.0f;
+            o[q][1] = in && c + 1 < cells ? G.ox[c] : 0.0f;
+            o[q][2] = in && c >= sy ? G.oy[c - sy] : 0.0f;
+            o[q][3] = in && c + sy < cells ? G.oy[c] : 0.0f;
+            o[q][4] = in && c >= sz ? G.oz[c - sz] : 0.0f;
+            o[q][5] = in && c + sz < cells ? G.oz[c] : 0.0f;
+        }
+    }
+    __device__ __forceinline__ float apply(int q, int c, int sy, int sz, int cells,
+                                           const float *v) const {
+        float s = diag[q] * v[c];
+        s = fmaf(o[q][0], v[max(c - 1, 0)], s);
+        s = fmaf(o[q][1], v[min(c + 1, cells - 1)], s);
+        s = fmaf(o[q][2], v[c >= sy ? c - sy : c], s);
+        s = fmaf(o[q][3], v[c + sy < cells ? c + sy : c], s);
+        s = fmaf(o[q][4], v[c >= sz ? c - sz : c], s);
+        s = fmaf(o[q][5], v[c + sz < cells ? c + sz : c], s);
+        return s;
+    }
+};
+
+#define OWN_CELLS(S, q, c)                                                            \
+    _Pragma("unroll") for (int q = 0, c = tid; q < kMgOwn; ++q, c += kMgSmallThreads) \
+        if (c < (S).cells)
+
+// The rest of the cycle below the large levels, in one CTA: the vectors of all
+// small levels in shared memory, the first one's operator in registers and the
+// others' in shared memory (16^3 cells and below: 64 KB), the passes separated
+// by the CTA's barrier; the coarsest level keeps each cell's operator in
+// registers for its sweeps.  Cells that are not fluid have wd = b = 0 and only
+// zero couplings: they are computed like the others, and stay finite.  (Launched one by one, the three smallest levels of 128^3 took
 // 38 us a cycle; a cluster of 8 CTAs on data in L2 took 26 us for the two
 // smallest.)
 __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
@@ -471,23 +514,31 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
     auto level = [&](int l) {  // the level's place: levels follow one another
         SmallLevel S;
         int at = 0;
-        for (int k = 0; k < l; ++k) at += (int)M.L[k].cells * kMgWords;
+        for (int k = 0; k < l; ++k) at += (int)M.L[k].cells * (k == 0 ? 3 : kMgWords);
         S.n0 = M.L[l].n[0];
         S.n1 = M.L[l].n[1];
         S.n2 = M.L[l].n[2];
         S.cells = (int)M.L[l].cells;
         float *p = s_mg + at;
-        S.diag = p;
-        S.wd = p + S.cells;
-        S.ox = p + 2 * S.cells;
-        S.oy = p + 3 * S.cells;
-        S.oz = p + 4 * S.cells;
-        S.x = p + 5 * S.cells;
-        S.b = p + 6 * S.cells;
-        S.t = p + 7 * S.cells;
+        S.x = p;
+        S.b = p + S.cells;
+        S.t = p + 2 * S.cells;
+        S.diag = p + 3 * S.cells;  // these not on the first of several levels
+        S.wd = p + 4 * S.cells;
+        S.ox = p + 5 * S.cells;
+        S.oy = p + 6 * S.cells;
+        S.oz = p + 7 * S.cells;
         return S;
     };
-    for (int l = 0; l <= top; ++l) {
+    // the first level's operator: in registers, but for a cycle of that level alone
+    OwnCells own;
+    if (top > 0) {
+        own.load(M.L[0], tid);
+        const SmallLevel S = level(0);
+        for (int c = tid; c < S.cells; c += kMgSmallThreads)
+            S.b[c] = M.L[0].fluid[c] ? M.L[0].b[c] : 0.0f;
+    }
+    for (int l = top > 0 ? 1 : 0; l <= top; ++l) {
         const MgLevel &G = M.L[l];
         const SmallLevel S = level(l);
         for (int c = tid; c < S.cells; c += kMgSmallThreads) {
@@ -514,12 +565,22 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
     for (int l = 0; l < top; ++l) {
         const SmallLevel S = level(l), C = level(l + 1);
         // two sweeps from 0 (t: the first), the residual (t), its sums over the children
-        for (int c = tid; c < S.cells; c += kMgSmallThreads) S.t[c] = S.wd[c] * S.b[c];
-        __syncthreads();
-        for (int c = tid; c < S.cells; c += kMgSmallThreads)
-            S.x[c] = fmaf(S.wd[c], S.b[c] - S.apply(c, S.t), S.t[c]);
-        __syncthreads();
-        for (int c = tid; c < S.cells; c += kMgSmallThreads) S.t[c] = S.b[c] - S.apply(c, S.x);
+        if (l == 0) {
+            const int sy = S.n0, sz = S.n0 * S.n1;
+            OWN_CELLS(S, q, c) S.t[c] = own.wd[q] * S.b[c];
+            __syncthreads();
+            OWN_CELLS(S, q, c)
+                S.x[c] = fmaf(own.wd[q], S.b[c] - own.apply(q, c, sy, sz, S.cells, S.t), S.t[c]);
+            __syncthreads();
+            OWN_CELLS(S, q, c) S.t[c] = S.b[c] - own.apply(q, c, sy, sz, S.cells, S.x);
+        } else {
+            for (int c = tid; c < S.cells; c += kMgSmallThreads) S.t[c] = S.wd[c] * S.b[c];
+            __syncthreads();
+            for (int c = tid; c < S.cells; c += kMgSmallThreads)
+                S.x[c] = fmaf(S.wd[c], S.b[c] - S.apply(c, S.t), S.t[c]);
+            __syncthreads();
+            for (int c = tid; c < S.cells; c += kMgSmallThreads) S.t[c] = S.b[c] - S.apply(c, S.x);
+        }
         __syncthreads();
         for (int cc = tid; cc < C.cells; cc += kMgSmallThreads) {
             const int I = cc % C.n0, J = (cc / C.n0) % C.n1, K = cc / (C.n0 * C.n1);
@@ -584,16 +645,26 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
             S.x[c] += C.x[((k >> 1) * C.n1 + (j >> 1)) * C.n0 + (i >> 1)];
         }
         __syncthreads();
-        for (int c = tid; c < S.cells; c += kMgSmallThreads)
-            S.t[c] = fmaf(S.wd[c], S.b[c] - S.apply(c, S.x), S.x[c]);
-        __syncthreads();
-        for (int c = tid; c < S.cells; c += kMgSmallThreads)
-            S.x[c] = fmaf(S.wd[c], S.b[c] - S.apply(c, S.t), S.t[c]);
+        if (l == 0) {
+            const int sy = S.n0, sz = S.n0 * S.n1;
+            OWN_CELLS(S, q, c)
+                S.t[c] = fmaf(own.wd[q], S.b[c] - own.apply(q, c, sy, sz, S.cells, S.x), S.x[c]);
+            __syncthreads();
+            OWN_CELLS(S, q, c)
+                S.x[c] = fmaf(own.wd[q], S.b[c] - own.apply(q, c, sy, sz, S.cells, S.t), S.t[c]);
+        } else {
+            for (int c = tid; c < S.cells; c += kMgSmallThreads)
+                S.t[c] = fmaf(S.wd[c], S.b[c] - S.apply(c, S.x), S.x[c]);
+            __syncthreads();
+            for (int c = tid; c < S.cells; c += kMgSmallThreads)
+                S.x[c] = fmaf(S.wd[c], S.b[c] - S.apply(c, S.t), S.t[c]);
+        }
         __syncthreads();
     }
     const SmallLevel S = level(0);
     for (int c = tid; c < S.cells; c += kMgSmallThreads) M.L[0].x[c] = S.x[c];
 }
+#undef OWN_CELLS
 
 // b . x = r . z over the fluid cells, for a one-level cycle.
 __global__ void __launch_bounds__(kPcgThreads) k_mg_dot(MgLevel L, PcgBuffers B, int odd) {
@@ -783,9 +854,10 @@ static cudaError_t mg_vcycle(const Multigrid &M, const PcgBuffers &B, int odd, i
     const int from = top > 0 ? large : 0;
     S.levels = M.levels - from;
     for (int l = 0; l < S.levels; ++l) S.L[l] = M.L[from + l];
-    int64_t cells = 0;
-    for (int l = 0; l < S.levels; ++l) cells += S.L[l].cells;
-    const int smem = (int)(cells * kMgWords * (int64_t)sizeof(float));
+    int64_t words = 0;  // the first of several levels: its vectors alone
+    for (int l = 0; l < S.levels; ++l)
+        words += S.L[l].cells * (l == 0 && S.levels > 1 ? 3 : kMgWords);
+    const int smem = (int)(words * (int64_t)sizeof(float));
     const cudaError_t e = cudaFuncSetAttribute(k_mg_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     k_mg_small<<<1, kMgSmallThreads, smem, s>>>(S);
