@@ -28,7 +28,7 @@
 // all smaller levels run in one CTA from shared memory.  The working set stays in L2
 // (60 MB at 128^3); a pass is bound by its loads' latency and by launching.
 // The grid update of 128^3 with 476 thousand fluid cells, 24 iterations, takes
-// 2.23 ms; 4.68 ms before, with a thread per cell of the box on every level,
+// 2.20 ms; 4.68 ms before, with a thread per cell of the box on every level,
 // 23 launches per iteration and the coarsest level's operator read from memory
 // on each of its 32 sweeps.
 #include <algorithm>
@@ -502,11 +502,11 @@ struct OwnCells {
 // The rest of the cycle below the large levels, in one CTA: the vectors of all
 // small levels in shared memory, the first one's operator in registers and the
 // others' in shared memory (16^3 cells and below: 64 KB), the passes separated
-// by the CTA's barrier; the coarsest level keeps each cell's operator in
-// registers for its sweeps.  Cells that are not fluid have wd = b = 0 and only
-// zero couplings: they are computed like the others, and stay finite.  (Launched one by one, the three smallest levels of 128^3 took
-// 38 us a cycle; a cluster of 8 CTAs on data in L2 took 26 us for the two
-// smallest.)
+// by the CTA's barrier; the coarsest level keeps each cell's operator and value
+// in registers for its sweeps.  Cells that are not fluid have wd = b = 0 and
+// only zero couplings: they are computed like the others, and stay finite.
+// (Launched one by one, the three smallest levels of 128^3 took 38 us a cycle;
+// a cluster of 8 CTAs on data in L2 took 26 us for the two smallest.)
 __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
     extern __shared__ float s_mg[];
     const int tid = (int)threadIdx.x;
@@ -530,13 +530,19 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
         S.oz = p + 7 * S.cells;
         return S;
     };
-    // the first level's operator: in registers, but for a cycle of that level alone
+    // The first of several levels: b first, its two loads independent (b of a
+    // cell that is not fluid may be anything), then the other levels, then the
+    // operator into registers, in flight until the first pass.
     OwnCells own;
+    float b0[kMgOwn];
+    uint8_t f0[kMgOwn];
     if (top > 0) {
-        own.load(M.L[0], tid);
-        const SmallLevel S = level(0);
-        for (int c = tid; c < S.cells; c += kMgSmallThreads)
-            S.b[c] = M.L[0].fluid[c] ? M.L[0].b[c] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < kMgOwn; ++q) {
+            const int c = min(tid + q * kMgSmallThreads, (int)M.L[0].cells - 1);
+            b0[q] = M.L[0].b[c];
+            f0[q] = M.L[0].fluid[c];
+        }
     }
     for (int l = top > 0 ? 1 : 0; l <= top; ++l) {
         const MgLevel &G = M.L[l];
@@ -560,6 +566,11 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
                 S.oz[c] = fl && k + 1 < S.n2 && G.fluid[c + S.n0 * S.n1] ? -1.0f : 0.0f;
             }
         }
+    }
+    if (top > 0) {
+        const SmallLevel S = level(0);
+        OWN_CELLS(S, q, c) S.b[c] = f0[q] ? b0[q] : 0.0f;
+        own.load(M.L[0], tid);
     }
     __syncthreads();
     for (int l = 0; l < top; ++l) {
@@ -600,7 +611,7 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
         const SmallLevel S = level(top);
         const int c = tid, sy = S.n0, sz = S.n0 * S.n1;
         const bool in = c < S.cells;
-        float o[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, diag = 0.0f, wd = 0.0f, b = 0.0f;
+        float o[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, diag = 0.0f, wd = 0.0f, b = 0.0f, v = 0.0f;
         int m[6] = {c, c, c, c, c, c};
         if (in) {
             const int st[3] = {1, sy, sz};
@@ -627,10 +638,10 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
                 const float *from = (it & 1) ? S.t : S.x;
                 float *to = (it & 1) ? S.x : S.t;
                 if (in) {
-                    float s = diag * from[c];
+                    float s = diag * v;
 #pragma unroll
                     for (int e = 0; e < 6; ++e) s = fmaf(o[e], from[m[e]], s);
-                    to[c] = fmaf(wd, b - s, from[c]);
+                    to[c] = v = fmaf(wd, b - s, v);
                 }
                 // the sweeps' own barrier: only the warps that take part
                 asm volatile("bar.sync 1, %0;" ::"n"(kMgCoarsest) : "memory");
@@ -640,9 +651,18 @@ __global__ void __launch_bounds__(kMgSmallThreads) k_mg_small(MgSmall M) {
     }
     for (int l = top - 1; l >= 0; --l) {
         const SmallLevel S = level(l), C = level(l + 1);
-        for (int c = tid; c < S.cells; c += kMgSmallThreads) {
-            const int i = c % S.n0, j = (c / S.n0) % S.n1, k = c / (S.n0 * S.n1);
-            S.x[c] += C.x[((k >> 1) * C.n1 + (j >> 1)) * C.n0 + (i >> 1)];
+        // two threads a coarse cell, four children each: the divisions of the
+        // index once for the four (a thread per child: 4,250 cycles of 32,000;
+        // with the loads of b and of the operator reordered 16.7 -> 15.0 us)
+        for (int u = tid; u < 2 * C.cells; u += kMgSmallThreads) {
+            const int up = u >= C.cells, cc = u - up * C.cells;
+            const int I = cc % C.n0, J = (cc / C.n0) % C.n1, K = cc / (C.n0 * C.n1);
+            const float x = C.x[cc];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int i = 2 * I + (q & 1), j = 2 * J + (q >> 1), k = 2 * K + up;
+                if (i < S.n0 && j < S.n1 && k < S.n2) S.x[(k * S.n1 + j) * S.n0 + i] += x;
+            }
         }
         __syncthreads();
         if (l == 0) {
