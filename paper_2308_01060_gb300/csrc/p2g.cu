@@ -5,16 +5,17 @@
 //
 // Work decomposition (no float atomics anywhere, so the result is
 // bit-identical from run to run):
-//   * one CTA per 8x8x4-cell tile, one warp per 4x4x2-cell block of it, one
-//     lane per cell.  Particles are in block-interleaved slot order (see
-//     sort.cu), so in round r the lanes read the r-th particle of their cell
-//     from one contiguous run of slots: coalesced loads, no reduction across
-//     lanes;
+//   * one CTA per 8x8x4-cell tile.  Two kernels fill its region (launch_p2g
+//     says which, p2g_chunks.cuh describes the other one); for 1, 4 and 8
+//     modes of a fluid there is one warp per 4x4x2-cell block, one lane per
+//     cell.  Particles are in block-interleaved slot order (see sort.cu), so
+//     in round r the lanes read the r-th particle of their cell from one
+//     contiguous run of slots: coalesced loads, no reduction across lanes;
 //   * a lane accumulates its cell's footprint on face grid A in registers:
 //     4 x 3 x 3 nodes (the particle's stencil is 3 nodes wide on every axis,
 //     but its lowest node along A is cell - 1 or cell), mass and momentum.
 //     The mode sum uses sum factorisation with the padded axis contracted
-//     last: 81 + 81 + 108 FMA per particle and component for 27 modes;
+//     last;
 //   * after the last round the warp adds the 32 cell footprints into its
 //     block region in 36 phases (one node offset per phase: distinct cells
 //     hit distinct nodes), then the CTA adds its 8 block regions into the
@@ -263,7 +264,7 @@ static cudaError_t reduce_tiles(const P2GArgs &P, float *gm[3], float *gp[3], fl
 // phases (a sheet holds its particles in few cells of a block) take the chunk
 // kernel, whose contraction keeps every lane busy; 1, 4 and 8 modes of a fluid
 // have too little contraction to pay for its exchange buffer: 460 us against
-// 408 (4 modes FP32) and 328 against 300 (8 modes FP16) on the fluids of 3.8
+// 372 (4 modes FP32) and 328 against 268 (8 modes FP16) on the fluids of 3.8
 // and 2.6 million particles, where 27 modes FP32 take 674 instead of 855.
 static cudaError_t launch_p2g(const P2GArgs &P, int R, int fmt, cudaStream_t s) {
     const int grid = (int)(P.nblocks / kP2GWarps);

@@ -1,13 +1,13 @@
 // p2g_kernel.cuh -- the per-particle pieces of the P2G transfer (Eqs 1-5,
-// 13, 15-19) used by the tile kernel of p2g_tiles.cuh: cp.async staging of a
-// particle, the sum-factorised accumulation into a lane's padded 4 x 3 x 3
-// footprint, and the slot of a lane's particle in a round.
+// 13, 15-19): the 1-D factors and Eq 12's affine map, which both P2G kernels
+// (p2g_tiles.cuh, p2g_chunks.cuh) use, and for the lane-per-cell one the
+// cp.async staging of a particle and the sum-factorised accumulation into a
+// lane's padded 4 x 3 x 3 footprint.
 #pragma once
 #include "cp_async.cuh"
 #include "p2g.cuh"
 
 namespace polypic {
-
 
 template <int A> struct TileReg {
     static constexpr int X = tile_x(A), Y = tile_y(A), Z = tile_z(A);
@@ -44,8 +44,8 @@ template <int A> __host__ __device__ constexpr int deg_z(int du, int dv, int dw)
 // ---------------------------------------------------------------- staging
 // Each lane prefetches its next particles with cp.async (4-byte copies) into
 // a private multi-stage buffer laid out [stage][value][lane] (conflict-free):
-// x, y, z, m, m_abs, s_p, the particle index, then the coefficient words: one
-// per mode for FP32, one per pair of modes for the 16-bit formats (whose
+// x, y, z, m, m_abs, s_p, then the coefficient words: one per mode for
+// FP32, one per pair of modes for the 16-bit formats (whose
 // words hold two codes).  With Eq 12's affine map (AFF) six more words
 // follow: the linear-mode coefficients of the two other components (their C
 // rows).
@@ -53,7 +53,7 @@ __host__ __device__ constexpr int coeff_words(int R, int FMT) {
     return FMT == POLYPIC_COEFF_F32 ? R : (R + 1) / 2;
 }
 template <int R, bool AFF = false, int FMT = POLYPIC_COEFF_F32> struct Stage {
-    static constexpr int kX = 0, kY = 1, kZ = 2, kM = 3, kMabs = 4, kScale = 5, kIdx = 6, kC = 7;
+    static constexpr int kX = 0, kY = 1, kZ = 2, kM = 3, kMabs = 4, kScale = 5, kC = 6;
     static constexpr int kL = kC + coeff_words(R, FMT);
     static constexpr int NV = kL + (AFF ? 6 : 0);
 };
