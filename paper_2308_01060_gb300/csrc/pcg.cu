@@ -311,39 +311,48 @@ __global__ void __launch_bounds__(kPcgThreads) k_list_write(MgLevel L, int c0, i
 // word on the finest level (elsewhere its parity bits alone); v(m, e): the
 // vector at cell m, whose coarse cell is e cells from c's; csy, csz: the
 // coarse strides.  A zero coupling (also the one that a row's end stores
-// towards the next row) reads nothing.
-template <bool TOP, class V>
+// towards the next row) adds nothing.  AHEAD: v may be read at any cell of the
+// box, so that its loads wait for neither the info word nor the couplings
+// (what a cell that is not fluid holds is read and not used).  With the lists
+// and vectors read by __ldg, which lets a pass's next cell start before this
+// one's store, an iteration at 128^3 goes from 88 to 85 us.
+template <bool TOP, bool AHEAD, class V>
 __device__ __forceinline__ float list_apply(const MgLevel &L, int c, unsigned w, int csy, int csz,
                                             const V &v) {
-    const int sy = L.n[0], sz = L.n[0] * L.n[1];
+    const int sy = L.n[0], sz = L.n[0] * L.n[1], end = (int)L.cells - 1;
     const int px = (w >> 10) & 1, py = (w >> 11) & 1, pz = (w >> 12) & 1;
+    const int m[6] = {c - 1, c + 1, c - sy, c + sy, c - sz, c + sz};
+    const int e[6] = {px - 1, px, py ? 0 : -csy, py ? csy : 0, pz ? 0 : -csz, pz ? csz : 0};
+    float n[6];
+    if constexpr (AHEAD) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) n[q] = v(q & 1 ? min(m[q], end) : max(m[q], 0), 0);
+    }
     if constexpr (TOP) {
         float s = info_diag(w) * v(c, 0);
-        if (w & 1u) s -= v(c - 1, px - 1);
-        if (w & 2u) s -= v(c + 1, px);
-        if (w & 4u) s -= v(c - sy, py ? 0 : -csy);
-        if (w & 8u) s -= v(c + sy, py ? csy : 0);
-        if (w & 16u) s -= v(c - sz, pz ? 0 : -csz);
-        if (w & 32u) s -= v(c + sz, pz ? csz : 0);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            if constexpr (AHEAD) s = w & (1u << q) ? s - n[q] : s;
+            else if (w & (1u << q)) s -= v(m[q], e[q]);
+        }
         return s;
     } else {
-        const float xm = c >= 1 ? L.ox[c - 1] : 0.0f, xp = L.ox[c];
-        const float ym = c >= sy ? L.oy[c - sy] : 0.0f, yp = L.oy[c];
-        const float zm = c >= sz ? L.oz[c - sz] : 0.0f, zp = L.oz[c];
-        float s = L.diag[c] * v(c, 0);
-        if (xm != 0.0f) s = fmaf(xm, v(c - 1, px - 1), s);
-        if (xp != 0.0f) s = fmaf(xp, v(c + 1, px), s);
-        if (ym != 0.0f) s = fmaf(ym, v(c - sy, py ? 0 : -csy), s);
-        if (yp != 0.0f) s = fmaf(yp, v(c + sy, py ? csy : 0), s);
-        if (zm != 0.0f) s = fmaf(zm, v(c - sz, pz ? 0 : -csz), s);
-        if (zp != 0.0f) s = fmaf(zp, v(c + sz, pz ? csz : 0), s);
+        const float o[6] = {c >= 1 ? __ldg(L.ox + c - 1) : 0.0f,   __ldg(L.ox + c),
+                            c >= sy ? __ldg(L.oy + c - sy) : 0.0f, __ldg(L.oy + c),
+                            c >= sz ? __ldg(L.oz + c - sz) : 0.0f, __ldg(L.oz + c)};
+        float s = __ldg(L.diag + c) * v(c, 0);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            if constexpr (AHEAD) s = o[q] != 0.0f ? fmaf(o[q], n[q], s) : s;
+            else if (o[q] != 0.0f) s = fmaf(o[q], v(m[q], e[q]), s);
+        }
         return s;
     }
 }
 
 template <bool TOP> __device__ __forceinline__ float list_wd(const MgLevel &L, int c, unsigned w) {
     if constexpr (TOP) return kMgOmega / info_diag(w);
-    else return L.wd[c];
+    else return __ldg(L.wd + c);
 }
 
 #define LIST_CELLS(L, t) \
@@ -353,12 +362,12 @@ template <bool TOP> __device__ __forceinline__ float list_wd(const MgLevel &L, i
 // Two damped-Jacobi sweeps from x = 0: x1 = w b / D, x = x1 + w (b - A x1) / D.
 // On the finest level x1 is in L.t (k_setup and k_update leave it there).
 template <bool TOP> __global__ void __launch_bounds__(kPcgThreads) k_mg_pre(MgLevel L) {
-    auto x1 = [&](int m, int) { return TOP ? L.t[m] : L.wd[m] * L.b[m]; };
+    auto x1 = [&](int m, int) { return TOP ? __ldg(L.t + m) : __ldg(L.wd + m) * __ldg(L.b + m); };
     LIST_CELLS(L, t) {
-        const int c = (int)L.idx[t];
-        const unsigned w = TOP ? L.info[c] : 0u;
-        const float ax = list_apply<TOP>(L, c, w, 0, 0, x1);
-        L.x[c] = fmaf(list_wd<TOP>(L, c, w), L.b[c] - ax, x1(c, 0));
+        const int c = (int)__ldg(L.idx + t);
+        const unsigned w = TOP ? __ldg(L.info + c) : 0u;
+        const float ax = list_apply<TOP, true>(L, c, w, 0, 0, x1);
+        L.x[c] = fmaf(list_wd<TOP>(L, c, w), __ldg(L.b + c) - ax, x1(c, 0));
     }
 }
 
@@ -367,13 +376,13 @@ template <bool TOP> __global__ void __launch_bounds__(kPcgThreads) k_mg_pre(MgLe
 // the children's order.
 template <bool TOP>
 __global__ void __launch_bounds__(kPcgThreads) k_mg_restrict(MgLevel F, MgLevel C, bool list) {
-    auto xf = [&](int m, int) { return F.x[m]; };
+    auto xf = [&](int m, int) { return __ldg(F.x + m); };
     const int64_t total = 8 * (list ? (int64_t)*C.count : C.cells);
     const int lane = threadIdx.x & 31;
     const unsigned group = 0xffu << (lane & 24);
     for (int64_t u = (int64_t)blockIdx.x * kPcgThreads + threadIdx.x; u < total;
          u += (int64_t)gridDim.x * kPcgThreads) {
-        const int64_t cc = list ? (int64_t)C.idx[u >> 3] : u >> 3;
+        const int64_t cc = list ? (int64_t)__ldg(C.idx + (u >> 3)) : u >> 3;
         const int q = (int)(u & 7);
         int I, J, K;
         mg_ijk(C, cc, I, J, K);
@@ -381,9 +390,9 @@ __global__ void __launch_bounds__(kPcgThreads) k_mg_restrict(MgLevel F, MgLevel 
         float r = 0.0f;
         if (i < F.n[0] && j < F.n[1] && k < F.n[2]) {
             const int c = (k * F.n[1] + j) * F.n[0] + i;
-            const unsigned w = TOP ? F.info[c] : 0u;
-            if (TOP ? (w & kInfoFluid) != 0 : F.fluid[c] != 0)
-                r = F.b[c] - list_apply<TOP>(F, c, w, 0, 0, xf);
+            const unsigned w = TOP ? __ldg(F.info + c) : 0u;
+            const float a = __ldg(F.b + c) - list_apply<TOP, true>(F, c, w, 0, 0, xf);
+            if (TOP ? (w & kInfoFluid) != 0 : __ldg(F.fluid + c) != 0) r = a;
         }
         float s = 0.0f;
 #pragma unroll
@@ -398,18 +407,18 @@ template <bool TOP>
 __global__ void __launch_bounds__(kPcgThreads) k_mg_post(MgLevel F, MgLevel C) {
     const int csy = C.n[0], csz = C.n[0] * C.n[1];
     LIST_CELLS(F, t) {
-        const int c = (int)F.idx[t], pc = (int)F.par[t];
+        const int c = (int)__ldg(F.idx + t), pc = (int)__ldg(F.par + t);
         unsigned w;
         if constexpr (TOP) {
-            w = F.info[c];
+            w = __ldg(F.info + c);
         } else {
             int i, j, k;
             mg_ijk(F, c, i, j, k);
             w = ((i & 1) << 10) | ((j & 1) << 11) | ((k & 1) << 12);
         }
-        auto xp = [&](int m, int e) { return F.x[m] + C.x[pc + e]; };
-        const float ax = list_apply<TOP>(F, c, w, csy, csz, xp);
-        F.t[c] = fmaf(list_wd<TOP>(F, c, w), F.b[c] - ax, xp(c, 0));
+        auto xp = [&](int m, int e) { return __ldg(F.x + m) + __ldg(C.x + pc + e); };
+        const float ax = list_apply<TOP, false>(F, c, w, csy, csz, xp);
+        F.t[c] = fmaf(list_wd<TOP>(F, c, w), __ldg(F.b + c) - ax, xp(c, 0));
     }
 }
 
@@ -417,13 +426,13 @@ __global__ void __launch_bounds__(kPcgThreads) k_mg_post(MgLevel F, MgLevel C) {
 // forms b . x = r . z for CG.
 template <bool TOP>
 __global__ void __launch_bounds__(kPcgThreads) k_mg_sweep(MgLevel L, PcgBuffers B, int odd) {
-    auto tv = [&](int m, int) { return L.t[m]; };
+    auto tv = [&](int m, int) { return __ldg(L.t + m); };
     double rz = 0.0;
     LIST_CELLS(L, t) {
-        const int c = (int)L.idx[t];
-        const unsigned w = TOP ? L.info[c] : 0u;
-        const float b = L.b[c];
-        const float out = fmaf(list_wd<TOP>(L, c, w), b - list_apply<TOP>(L, c, w, 0, 0, tv), L.t[c]);
+        const int c = (int)__ldg(L.idx + t);
+        const unsigned w = TOP ? __ldg(L.info + c) : 0u;
+        const float b = __ldg(L.b + c);
+        const float out = fmaf(list_wd<TOP>(L, c, w), b - list_apply<TOP, true>(L, c, w, 0, 0, tv), tv(c, 0));
         if (TOP) rz += (double)b * (double)out;
         L.x[c] = out;
     }
@@ -780,12 +789,12 @@ __global__ void __launch_bounds__(kPcgThreads) k_apply(MgLevel L, PcgBuffers B, 
         const double rz = B.scal[kRz + odd], prev = B.scal[kRz + (odd ^ 1)];
         beta = prev == 0.0 ? 0.0f : (float)(rz / prev);
     }
-    auto dn = [&](int m, int) { return fmaf(beta, d_in[m], B.z[m]); };
+    auto dn = [&](int m, int) { return fmaf(beta, __ldg(d_in + m), __ldg(B.z + m)); };
     double pap = 0.0;
     LIST_CELLS(L, t) {
-        const int c = (int)L.idx[t];
+        const int c = (int)__ldg(L.idx + t);
         const float dc = dn(c, 0);
-        const float s = list_apply<true>(L, c, L.info[c], 0, 0, dn);
+        const float s = list_apply<true, true>(L, c, __ldg(L.info + c), 0, 0, dn);
         d_out[c] = dc;
         B.Ap[c] = s;
         pap += (double)dc * (double)s;
