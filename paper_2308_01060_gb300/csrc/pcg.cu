@@ -813,13 +813,26 @@ __global__ void __launch_bounds__(kPcgThreads) k_update(MgLevel L, PcgBuffers B,
     const double pap = B.scal[kPAp], rz = B.scal[kRz + odd];
     const float alpha = pap != 0.0 ? (float)(rz / pap) : 0.0f;
     double rr = 0.0;
-    LIST_CELLS(L, t) {
-        const int c = (int)L.idx[t];
-        B.x[c] = fmaf(alpha, d[c], B.x[c]);
-        const float r = fmaf(-alpha, B.Ap[c], B.r[c]);
-        B.r[c] = r;
-        B.Ap[c] = (kMgOmega / info_diag(L.info[c])) * r;
-        rr += (double)r * (double)r;
+    const uint32_t n = *L.count, step = gridDim.x * kPcgThreads;
+    for (uint32_t t = blockIdx.x * kPcgThreads + threadIdx.x; t < n; t += 2 * step) {
+        // two cells at a time, their loads ahead of either's stores: 9.1 -> 8.1 us at 128^3
+        const bool two = step < n - t;
+        const int c[2] = {(int)__ldg(L.idx + t), (int)__ldg(L.idx + (two ? t + step : t))};
+        float x[2], r[2], wd[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            x[q] = fmaf(alpha, __ldg(d + c[q]), B.x[c[q]]);
+            r[q] = fmaf(-alpha, B.Ap[c[q]], B.r[c[q]]);
+            wd[q] = kMgOmega / info_diag(__ldg(L.info + c[q]));
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q == 1 && !two) break;
+            B.x[c[q]] = x[q];
+            B.r[c[q]] = r[q];
+            B.Ap[c[q]] = wd[q] * r[q];
+            rr += (double)r[q] * (double)r[q];
+        }
     }
     rr = block_sum(rr);
     if (threadIdx.x == 0) B.rr[blockIdx.x] = rr;
