@@ -8,9 +8,8 @@
 // solved by conjugate gradients with FP32 vectors and FP64 dot products and
 // norms (two-stage deterministic reductions), preconditioned by one
 // multigrid V-cycle; then v_a -= dt / (rho dx) (p_hi - p_lo) on every non-wall
-// face next to a fluid cell.  alpha and beta are formed on the device by the
-// kernels that use them; the host reads the residual norm every kCheckEvery
-// iterations.
+// face next to a fluid cell.  alpha and beta are formed on the device with the
+// dot products; the host reads the residual norm every kCheckEvery iterations.
 //
 // The V-cycle (an aggregation multigrid): a coarse cell is the 2x2x2 block of
 // fine cells, fluid if any child is; the coarse operator is the Galerkin
@@ -28,7 +27,7 @@
 // all smaller levels run in one CTA from shared memory.  The working set stays in L2
 // (60 MB at 128^3); a pass is bound by its loads' latency and by launching.
 // The grid update of 128^3 with 476 thousand fluid cells, 24 iterations, takes
-// 2.20 ms; 4.68 ms before, with a thread per cell of the box on every level,
+// 2.09 ms; 4.68 ms before, with a thread per cell of the box on every level,
 // 23 launches per iteration and the coarsest level's operator read from memory
 // on each of its 32 sweeps.
 #include <algorithm>
@@ -51,8 +50,9 @@ struct PcgBuffers {
     uint32_t *arrived;  // blocks of the running kernel that have left their sum
 };
 
-// scal[]: |r|^2 and |b|^2 for the host, d . Ap, and r . z by the iteration's parity
-enum { kRr = 0, kBb = 1, kPAp = 2, kRz = 3 };
+// scal[]: |r|^2 and |b|^2 for the host, r . z by the iteration's parity, and
+// CG's alpha and beta (rounded to FP32)
+enum { kRr = 0, kBb = 1, kRz = 3, kAlpha = 5, kBeta = 6 };
 
 __device__ __forceinline__ int64_t cidx(const GridGeom &g, int i, int j, int k) {
     return ((int64_t)k * g.n[1] + j) * g.n[0] + i;
@@ -85,8 +85,12 @@ __device__ __forceinline__ double block_total(const double *sums, int nb) {
 
 // Sum of `a` over the grid into *out: the block that arrives last adds the
 // block sums, in block order whatever the order of arrival, so that the total
-// needs no launch of its own and no block waits for another.
-__device__ __forceinline__ void grid_sum(double a, const PcgBuffers &B, double *out) {
+// needs no launch of its own and no block waits for another.  Its thread 0
+// also calls done(total): the FP64 quotients of CG are formed there, once,
+// instead of by every thread that uses them (k_apply 10.9 -> 9.7, k_update 8.0
+// -> 6.6, k_mg_sweep 8.3 -> 8.9 us at 128^3).
+template <class Done>
+__device__ __forceinline__ void grid_sum(double a, const PcgBuffers &B, const Done &done) {
     __shared__ bool last;
     a = block_sum(a);
     if (threadIdx.x == 0) {
@@ -101,7 +105,15 @@ __device__ __forceinline__ void grid_sum(double a, const PcgBuffers &B, double *
     double t = 0.0;
     for (int i = threadIdx.x; i < (int)gridDim.x; i += kPcgThreads) t += sums[i];
     t = block_sum(t);
-    if (threadIdx.x == 0) *out = t;
+    if (threadIdx.x == 0) done(t);
+}
+
+// r . z of iteration `odd`, and beta of the direction that follows (0 if the
+// previous r . z is 0; the first direction has none and ignores it).
+__device__ __forceinline__ void put_rz(const PcgBuffers &B, int odd, double rz) {
+    const double prev = B.scal[kRz + (odd ^ 1)];
+    B.scal[kRz + odd] = rz;
+    B.scal[kBeta] = prev == 0.0 ? 0.0f : (float)(rz / prev);
 }
 
 __global__ void __launch_bounds__(kPcgThreads) k_total(const double *sums, int nb, double *out) {
@@ -440,7 +452,7 @@ __global__ void __launch_bounds__(kPcgThreads) k_mg_sweep(MgLevel L, PcgBuffers 
         if (TOP) rz += (double)b * (double)out;
         L.x[c] = out;
     }
-    if constexpr (TOP) grid_sum(rz, B, B.scal + kRz + odd);
+    if constexpr (TOP) grid_sum(rz, B, [&](double t) { put_rz(B, odd, t); });
 }
 
 // ---------------------------------------------------------------- small levels
@@ -706,7 +718,7 @@ __global__ void __launch_bounds__(kPcgThreads) k_mg_dot(MgLevel L, PcgBuffers B,
         const uint32_t c = L.idx[t];
         rz += (double)L.b[c] * (double)L.x[c];
     }
-    grid_sum(rz, B, B.scal + kRz + odd);
+    grid_sum(rz, B, [&](double t) { put_rz(B, odd, t); });
 }
 
 struct Multigrid {
@@ -779,7 +791,7 @@ __global__ void __launch_bounds__(kPcgThreads) k_setup(GridGeom g, int64_t num_k
         B.d[c] = 0.0f;
         bb += (double)b * (double)b;
     }
-    grid_sum(bb, B, B.scal + kBb);
+    grid_sum(bb, B, [&](double t) { B.scal[kBb] = t; });
 }
 
 // The new direction and its product with A in one pass: d_out = z + beta d_in
@@ -788,11 +800,7 @@ __global__ void __launch_bounds__(kPcgThreads) k_setup(GridGeom g, int64_t num_k
 __global__ void __launch_bounds__(kPcgThreads) k_apply(MgLevel L, PcgBuffers B, int odd,
                                                        const float *d_in, float *d_out,
                                                        bool first) {
-    float beta = 0.0f;
-    if (!first) {
-        const double rz = B.scal[kRz + odd], prev = B.scal[kRz + (odd ^ 1)];
-        beta = prev == 0.0 ? 0.0f : (float)(rz / prev);
-    }
+    const float beta = first ? 0.0f : (float)B.scal[kBeta];
     auto dn = [&](int m, int) { return fmaf(beta, __ldg(d_in + m), __ldg(B.z + m)); };
     double pap = 0.0;
     LIST_CELLS(L, t) {
@@ -803,19 +811,20 @@ __global__ void __launch_bounds__(kPcgThreads) k_apply(MgLevel L, PcgBuffers B, 
         B.Ap[c] = s;
         pap += (double)dc * (double)s;
     }
-    grid_sum(pap, B, B.scal + kPAp);
+    grid_sum(pap, B, [&](double t) {  // alpha of the step along the direction
+        B.scal[kAlpha] = t != 0.0 ? (float)(B.scal[kRz + odd] / t) : 0.0f;
+    });
 }
 
 // The step along d, the residual and its block sums, and in Ap's place the
 // first sweep of the cycle that follows, w r / D.
-__global__ void __launch_bounds__(kPcgThreads) k_update(MgLevel L, PcgBuffers B, int odd,
+__global__ void __launch_bounds__(kPcgThreads) k_update(MgLevel L, PcgBuffers B,
                                                         const float *__restrict__ d) {
-    const double pap = B.scal[kPAp], rz = B.scal[kRz + odd];
-    const float alpha = pap != 0.0 ? (float)(rz / pap) : 0.0f;
+    const float alpha = (float)B.scal[kAlpha];
     double rr = 0.0;
     const uint32_t n = *L.count, step = gridDim.x * kPcgThreads;
     for (uint32_t t = blockIdx.x * kPcgThreads + threadIdx.x; t < n; t += 2 * step) {
-        // two cells at a time, their loads ahead of either's stores: 9.1 -> 8.1 us at 128^3
+        // two cells at a time, their loads ahead of either's stores (9.1 -> 8.1 us at 128^3)
         const bool two = step < n - t;
         const int c[2] = {(int)__ldg(L.idx + t), (int)__ldg(L.idx + (two ? t + step : t))};
         float x[2], r[2], wd[2];
@@ -930,7 +939,7 @@ static cudaError_t launch_batch(PcgBuffers &B, const Multigrid &M, int nb, int i
         const int odd = (it0 + b) & 1;
         float *d_in = odd ? B.d2 : B.d, *d_out = odd ? B.d : B.d2;
         k_apply<<<nb, kPcgThreads, 0, s>>>(M.L[0], B, odd, d_in, d_out, it0 + b == 0);
-        k_update<<<nb, kPcgThreads, 0, s>>>(M.L[0], B, odd, d_out);
+        k_update<<<nb, kPcgThreads, 0, s>>>(M.L[0], B, d_out);
         const cudaError_t e = mg_vcycle(M, B, odd ^ 1, nb, s);
         if (e != cudaSuccess) return e;
     }
