@@ -151,12 +151,12 @@ class ClockSampler:
 
 # ---------------------------------------------------------------- workload
 
-# DRAM bytes (read + write) per particle of one k_p2g_tiles<27, FP32> launch,
-# from a full ncu capture on the 96^3 dam break (1,557,376 particles: 537.2 MB
-# read, 13.8 MB written); P2G traffic grows in proportion to the particles, so
-# it scales to the 128^3 launch.  It must go back to None whenever the kernel
-# changes after that capture.
-P2G_TILES_DRAM_BYTES_PER_PARTICLE = (537.27232e6 + 13.886464e6) / 1557376
+# DRAM bytes (read + write) per particle of one k_p2g_chunks<27, FP32> launch,
+# from a full ncu capture on 96^3 with 1,555,632 particles, Poisson-distributed
+# over a quarter of the cells (589.1 MB read, 16.1 MB written); P2G traffic
+# grows in proportion to the particles, so it scales to the 128^3 launch.  It
+# must go back to None whenever the kernel changes after that capture.
+P2G_DRAM_BYTES_PER_PARTICLE = (589.093376e6 + 16.144896e6) / 1555632
 
 
 def block_cells(n: int):
@@ -1007,10 +1007,10 @@ def our_arm(args):
     roofline = {
         "bound": "hbm", "achieved": round(dom_gbs, 1), "peak": hbm, "unit": "GB/s",
         "frac": round(dom_gbs / hbm, 4),
-        "traffic": (round(P * P2G_TILES_DRAM_BYTES_PER_PARTICLE / 1e9, 4)
-                    if dominant == "p2g" and P2G_TILES_DRAM_BYTES_PER_PARTICLE else None),
-        "traffic_unit": "GB per launch (k_p2g_tiles only, scaled from a 96^3 capture)",
-        "kernel": "polypic_p2g call (k_p2g_tiles + k_p2g_reduce)" if dominant == "p2g"
+        "traffic": (round(P * P2G_DRAM_BYTES_PER_PARTICLE / 1e9, 4)
+                    if dominant == "p2g" and P2G_DRAM_BYTES_PER_PARTICLE else None),
+        "traffic_unit": "GB per launch (k_p2g_chunks only, scaled from a 96^3 capture)",
+        "kernel": "polypic_p2g call (k_p2g_chunks + k_p2g_reduce)" if dominant == "p2g"
         else "polypic_g2p (k_g2p_tiles)",
         "algorithmic_bytes_per_particle": p2g_b if dominant == "p2g" else g2p_b,
         "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"

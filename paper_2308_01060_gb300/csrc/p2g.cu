@@ -266,6 +266,8 @@ static cudaError_t reduce_tiles(const P2GArgs &P, float *gm[3], float *gp[3], fl
 // have too little contraction to pay for its exchange buffer: 460 us against
 // 372 (4 modes FP32) and 328 against 268 (8 modes FP16) on the fluids of 3.8
 // and 2.6 million particles, where 27 modes FP32 take 674 instead of 855.
+// These are spread fluids, cells filled unevenly; on freshly seeded ones (close
+// to 8 in every cell) 27 modes lose some 90 us by it, but no call knows that.
 static cudaError_t launch_p2g(const P2GArgs &P, int R, int fmt, cudaStream_t s) {
     const int grid = (int)(P.nblocks / kP2GWarps);
     if (P.affine) {  // Eq 12's affine map: FP32 coefficients, 4, 8 or 27 modes
