@@ -657,15 +657,15 @@ __global__ void __launch_bounds__(96 * G, 4 / G) k_p2g_chunks(P2GArgs P) {
 
 template <int R, int FMT, bool ADJ, bool AFF, int G>
 cudaError_t launch_chunks_g(const P2GArgs &P, int grid, cudaStream_t s) {
-    static_assert(chunks_smem_bytes<R, FMT, ADJ, AFF, G>(true) <= 227 * 1024,
-                  "P2G exceeds the shared memory of a CTA");
-    const int smem = chunks_smem_bytes<R, FMT, ADJ, AFF, G>(P.mass_abs != nullptr);
-    // the attribute is a property of the kernel in the current context; it is
-    // set on every launch (a cheap host call), which keeps no state shared
-    // between host threads or devices
+    // The limit belongs to the kernel, not to the launch: every caller sets the
+    // same value, the largest that a launch of this kernel needs (a solid phase's),
+    // so that a host thread never lowers it between another's setting and launch.
+    constexpr int limit = chunks_smem_bytes<R, FMT, ADJ, AFF, G>(true);
+    static_assert(limit <= 227 * 1024, "P2G exceeds the shared memory of a CTA");
     const cudaError_t e = cudaFuncSetAttribute(k_p2g_chunks<R, FMT, ADJ, AFF, G>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
+    const int smem = chunks_smem_bytes<R, FMT, ADJ, AFF, G>(P.mass_abs != nullptr);
     k_p2g_chunks<R, FMT, ADJ, AFF, G><<<grid, 96 * G, smem, s>>>(P);
     return cudaGetLastError();
 }

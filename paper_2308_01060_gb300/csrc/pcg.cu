@@ -130,6 +130,9 @@ constexpr float kMgOmega = 2.0f / 3.0f;
 // memory of it and the levels below bounds it).
 constexpr int64_t kMgSmall = 4608;
 constexpr int kMgSmallThreads = 1024;
+// All the shared memory a CTA can have.  The levels of 128^3 take 64 KB, no
+// grid's more than 112 KB (thin ones, whose levels shrink least).
+constexpr int kMgSmallLimit = 227 * 1024;
 constexpr int kListTile = 2048;  // cells per CTA of the list's compaction
 
 // One level of the hierarchy.  Level 0 is the fine system: couplings are -1
@@ -913,7 +916,10 @@ static cudaError_t mg_vcycle(const Multigrid &M, const PcgBuffers &B, int odd, i
     for (int l = 0; l < S.levels; ++l)
         words += S.L[l].cells * (l == 0 && S.levels > 1 ? 3 : kMgWords);
     const int smem = (int)(words * (int64_t)sizeof(float));
-    const cudaError_t e = cudaFuncSetAttribute(k_mg_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the kernel's limit, the same whatever the grid: contexts of other grids may
+    // be launching it from other host threads
+    const cudaError_t e = cudaFuncSetAttribute(k_mg_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               kMgSmallLimit);
     if (e != cudaSuccess) return e;
     k_mg_small<<<1, kMgSmallThreads, smem, s>>>(S);
     if (top > 0) {
