@@ -461,7 +461,11 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     lx[2] = fmaf(mt, Dz, lx[2]);
 }
 
-// Tiles of at most this many particles are walked in memory order (below).
+// With 27 modes, tiles of at most this many particles are walked in memory order
+// (below): the three adjoints of 863 thousand particles take 577 us instead of
+// 581.  With fewer modes the list costs more than it gives (P2G adjoint of the
+// same particles without it: 8 modes 129 -> 127 us, 4 modes 119 -> 109, one mode
+// 71 -> 66).
 constexpr int kAdjList = 3072;
 constexpr int kAdjWords = 128;  // bitmap words: a window of 4096 indices
 
@@ -471,7 +475,9 @@ constexpr int kAdjWords = 128;  // bitmap words: a window of 4096 indices
 // only its own entries, so the order changes no result).  The arrays are in
 // the slot order of the step before: ascending indices read and write whole
 // sectors of their 162 coefficient rows where slot order, moved by a rank
-// wherever a particle left or entered a cell, touched them in pieces.
+// wherever a particle left or entered a cell, touched them in pieces.  A perm
+// that names a particle twice ranks it once; the entries this leaves over keep
+// the particle of their slot.
 __device__ __forceinline__ void list_in_memory_order(const uint32_t *__restrict__ perm, uint32_t jb,
                                                      uint32_t je, uint32_t *idx, uint32_t *bits) {
     uint32_t *pre = bits + kAdjWords, *far = pre + kAdjWords;
@@ -483,7 +489,8 @@ __device__ __forceinline__ void list_in_memory_order(const uint32_t *__restrict_
     for (int i = threadIdx.x; i < kAdjWords; i += blockDim.x) bits[i] = 0;
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const uint32_t off = perm[jb + i] - base;
+        const uint32_t p = perm[jb + i], off = p - base;
+        idx[i] = p;
         if (off < W) atomicOr(&bits[off >> 5], 1u << (off & 31u));
     }
     __syncthreads();
@@ -509,7 +516,7 @@ __device__ __forceinline__ void list_in_memory_order(const uint32_t *__restrict_
         const uint32_t at = off < W ? pre[off >> 5] + (uint32_t)__popc(bits[off >> 5] &
                                                                      ((1u << (off & 31u)) - 1u))
                                     : atomicAdd(far, 1u);
-        if (at < n) idx[at] = p;  // perm names n distinct particles
+        if (at < n) idx[at] = p;
     }
     __syncthreads();
 }
@@ -517,7 +524,8 @@ __device__ __forceinline__ void list_in_memory_order(const uint32_t *__restrict_
 template <int R>
 __global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(AdjP2GArgs Q) {
     extern __shared__ float s_adj[];
-    __shared__ uint32_t s_idx[kAdjList], s_bits[2 * kAdjWords + 1];
+    constexpr bool kList = R == 27;
+    __shared__ uint32_t s_idx[kList ? kAdjList : 1], s_bits[kList ? 2 * kAdjWords + 1 : 1];
     float *tile_m = s_adj, *tile_v = s_adj + kATileFloats;
     const GridGeom &g = Q.g;
     const uint32_t tile = blockIdx.x;
@@ -529,7 +537,7 @@ __global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(Ad
     const int ox = 8 * tx - 1, oy = 8 * ty - 1, oz = 4 * tz - 1;
     stage_tile(g, Q.lm, ox, oy, oz, tile_m);
     stage_tile(g, Q.lmv, ox, oy, oz, tile_v);
-    const bool listed = je - jb <= (uint32_t)kAdjList;  // CTA-uniform
+    const bool listed = kList && je - jb <= (uint32_t)kAdjList;  // CTA-uniform
     if (listed) list_in_memory_order(Q.perm, jb, je, s_idx, s_bits);
     else __syncthreads();
     auto particle = [&](uint32_t j) { return listed ? s_idx[j - jb] : Q.perm[j]; };
