@@ -408,7 +408,8 @@ template <int R, int A>
 __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const ParticleAxes &pa,
                                                   const float *tile_m, const float *tile_v, int ox,
                                                   int oy, int oz, uint32_t p, float mt,
-                                                  const CoeffStage<R> &coef, float (&lx)[3]) {
+                                                  const CoeffStage<R> &coef,
+                                                  const CoeffStage<R> &old, float (&lx)[3]) {
     constexpr int D = axis_degrees(R);
     const Axis &ax = A == 0 ? pa.fce[0] : pa.ctr[0];
     const Axis &ay = A == 1 ? pa.fce[1] : pa.ctr[1];
@@ -438,21 +439,13 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     float lmv[3][3][3];
     read_stencil<A>(tile_v, lx0, ly0, lz0, lmv);
     contract_modes<R, D>(X, Y, Z, lmv, [&](int a, const float (&m)[D][D]) {
-        float old[D][D];
-        if (Q.accumulate) {  // the old values, loaded before the first store
-#pragma unroll
-            for (int b = 0; b < D; ++b)
-#pragma unroll
-                for (int cc = 0; cc < D; ++cc)
-                    old[b][cc] = has_mode(R, a, b, cc) ? cout[mode_index(a, b, cc) * cnt] : 0.0f;
-        }
 #pragma unroll
         for (int b = 0; b < D; ++b)
 #pragma unroll
             for (int cc = 0; cc < D; ++cc)
                 if (has_mode(R, a, b, cc))
                     cout[mode_index(a, b, cc) * cnt] =
-                        Q.accumulate ? fmaf(mt, m[b][cc], old[b][cc]) : mt * m[b][cc];
+                        Q.accumulate ? fmaf(mt, m[b][cc], old(a, b, cc)) : mt * m[b][cc];
     });
     // position terms of the momentum, through the modes
     adj_position<R, D, false>(X, dX, Y, dY, Z, dZ, lmv, coef, Dx, Dy, Dz);
@@ -542,8 +535,12 @@ __global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(Ad
     else __syncthreads();
     auto particle = [&](uint32_t j) { return listed ? s_idx[j - jb] : Q.perm[j]; };
     // software pipeline: the next particle's index, position and mass load
-    // while this one is computed, every component's coefficients one ahead
+    // while this one is computed, every component's coefficients one ahead, and
+    // its old outputs when they are added to (loaded where they are used, they
+    // cost a component three memory latencies)
     CoeffStage<R> coef(s_adj + 2 * kATileFloats);
+    CoeffStage<R> old(s_adj + 2 * kATileFloats + 2 * R * kAdjThreads);
+    const bool add = Q.accumulate;
     const int64_t cnt = Q.count;
     uint32_t j = jb + threadIdx.x;
     uint32_t pn = j < je ? particle(j) : 0u;
@@ -554,6 +551,7 @@ __global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(Ad
         nz = Q.x[2][pn];
         nm = Q.mass[pn] + (Q.mass_abs ? Q.mass_abs[pn] : 0.0f);
         coef.fill(false, Q.coeff + pn, cnt);
+        if (add) old.fill(false, Q.out_c + pn, cnt);
     }
     cp_async_commit();
     for (; j < je; j += kAdjThreads) {
@@ -571,12 +569,16 @@ __global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(Ad
         float lx[3] = {0.0f, 0.0f, 0.0f};
         auto component = [&](auto axis) {
             constexpr int A = decltype(axis)::value;
-            if (A < 2) coef.fill(true, Q.coeff + (int64_t)(A + 1) * R * cnt + p, cnt);
-            else if (more) coef.fill(true, Q.coeff + pn, cnt);
+            if (A < 2 || more) {
+                const int64_t at = A < 2 ? (int64_t)(A + 1) * R * cnt + p : (int64_t)pn;
+                coef.fill(true, Q.coeff + at, cnt);
+                if (add) old.fill(true, Q.out_c + at, cnt);
+            }
             cp_async_commit();
             cp_async_wait<1>();
-            if (pa.ok) p2g_adj_component<R, A>(Q, pa, tile_m, tile_v, ox, oy, oz, p, mt, coef, lx);
+            if (pa.ok) p2g_adj_component<R, A>(Q, pa, tile_m, tile_v, ox, oy, oz, p, mt, coef, old, lx);
             coef.next();
+            old.next();
         };
         component(std::integral_constant<int, 0>{});
         component(std::integral_constant<int, 1>{});
@@ -616,8 +618,11 @@ static cudaError_t launch_g2p_adjoint(const AdjG2PArgs &G, int64_t tiles, cudaSt
 
 template <int R>
 static cudaError_t launch_p2g_adjoint(const AdjP2GArgs &Q, int64_t tiles, cudaStream_t s) {
-    constexpr int smem = stage_bytes<R>() + 2 * kATileFloats * (int)sizeof(float);
-    const cudaError_t e = cudaFuncSetAttribute(k_p2g_adjoint<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    constexpr int tiles_bytes = 2 * kATileFloats * (int)sizeof(float);
+    constexpr int limit = tiles_bytes + 2 * stage_bytes<R>();  // the kernel's, whatever the call
+    static_assert(limit <= 200 * 1024, "the P2G adjoint exceeds the shared memory of a CTA");
+    const int smem = tiles_bytes + (Q.accumulate ? 2 : 1) * stage_bytes<R>();
+    const cudaError_t e = cudaFuncSetAttribute(k_p2g_adjoint<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
     k_p2g_adjoint<R><<<(int)tiles, kAdjThreads, smem, s>>>(Q);
     return cudaGetLastError();
