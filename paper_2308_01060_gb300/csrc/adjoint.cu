@@ -29,11 +29,26 @@
 namespace polypic {
 
 constexpr int kAdjThreads = 256;
-// Two CTAs an SM (128 registers) where that spills little: the G2P adjoint of
-// every mode set (27 modes with its scatter 319 -> 306 us on 863 thousand
-// particles) and the P2G adjoint of up to 8 modes (165 -> 130); the P2G adjoint
-// of 27 modes would spill 376 bytes a thread (262 -> 275 us).
-constexpr int p2g_adj_ctas(int R) { return R == 27 ? 1 : 2; }
+// CTAs of an SM that a gather's registers are limited for.  A phase of at most
+// one tile an SM (2048 particles each at 8 a cell) has no use for a second CTA,
+// only for the registers: on 119 thousand particles (33x29x45 cells) the P2G
+// adjoint of 8 modes takes 44 us with one and 53 with two, of 4 modes 37 and 47,
+// the G2P adjoint with its scatter of 27 modes 97 and 111.  Larger phases take
+// two (863 thousand particles: P2G adjoint of 8 modes 121 us, 157 with one; G2P
+// adjoint of 27 modes 307, 319 with one), but for the P2G adjoint of 27 modes,
+// which would spill 376 bytes a thread (262 -> 275 us).  One mode is small
+// enough for two and, above two tiles an SM, three (2.9 million particles: P2G
+// adjoint 210 -> 177 us; 364 thousand: 39 us with two, 51 with three).  A sparse
+// phase has more tiles than its count says, so the grid's count as well (62
+// thousand particles in half of 64^3, G2P adjoint of 27 modes: 133 us with one,
+// 121 with two; grids up to 48^3 are below the line).
+constexpr bool adj_few(int R, int64_t count, int64_t tiles) {
+    return count <= (R == 1 ? 2 : 1) * 152 * 2048 && tiles <= 152 * 4;
+}
+template <int R, bool FEW> constexpr int g2p_adj_ctas() { return (R == 1 ? 2 : 1) + (FEW ? 0 : 1); }
+template <int R, bool FEW> constexpr int p2g_adj_ctas() {
+    return R == 27 ? 1 : g2p_adj_ctas<R, FEW>();
+}
 template <int A> struct ATile {
     static constexpr int X = A == 0 ? 11 : 10, Y = A == 1 ? 11 : 10, Z = A == 2 ? 7 : 6;
     static constexpr int N = X * Y * Z;
@@ -338,8 +353,8 @@ __device__ __forceinline__ void g2p_adj_component(const AdjG2PArgs &G, const Par
     if (!clamped) lx[A] += lxo;
 }
 
-template <int R>
-__global__ void __launch_bounds__(kAdjThreads, 2) k_g2p_adjoint(AdjG2PArgs G) {
+template <int R, bool FEW>
+__global__ void __launch_bounds__(kAdjThreads, g2p_adj_ctas<R, FEW>()) k_g2p_adjoint(AdjG2PArgs G) {
     __shared__ float s_tile[kATileFloats];
     const GridGeom &g = G.g;
     const uint32_t tile = blockIdx.x;
@@ -423,19 +438,6 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     const int64_t cnt = Q.count;
     float *__restrict__ cout = Q.out_c + (int64_t)A * R * cnt + p;
     float Dx = 0.0f, Dy = 0.0f, Dz = 0.0f;
-    {  // position terms of the mass, through the weights
-        float lm[3][3][3];
-        read_stencil<A>(tile_m, lx0, ly0, lz0, lm);
-        float Wx[1][3], dWx[1][3], Wy[1][3], dWy[1][3], Wz[1][3], dWz[1][3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            Wx[0][k] = X[0][k]; dWx[0][k] = dX[0][k];
-            Wy[0][k] = Y[0][k]; dWy[0][k] = dY[0][k];
-            Wz[0][k] = Z[0][k]; dWz[0][k] = dZ[0][k];
-        }
-        auto one = [](int, int, int) { return 1.0f; };
-        adj_position<1, 1, false>(Wx, dWx, Wy, dWy, Wz, dWz, lm, one, Dx, Dy, Dz);
-    }
     float lmv[3][3][3];
     read_stencil<A>(tile_v, lx0, ly0, lz0, lmv);
     contract_modes<R, D>(X, Y, Z, lmv, [&](int a, const float (&m)[D][D]) {
@@ -449,9 +451,25 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     });
     // position terms of the momentum, through the modes
     adj_position<R, D, false>(X, dX, Y, dY, Z, dZ, lmv, coef, Dx, Dy, Dz);
-    lx[0] = fmaf(mt, Dx, lx[0]);
-    lx[1] = fmaf(mt, Dy, lx[1]);
-    lx[2] = fmaf(mt, Dz, lx[2]);
+    // position terms of the mass, through the weights (ahead of the momentum's:
+    // 1-5% slower), summed by themselves
+    float Mx = 0.0f, My = 0.0f, Mz = 0.0f;
+    {
+        float lm[3][3][3];
+        read_stencil<A>(tile_m, lx0, ly0, lz0, lm);
+        float Wx[1][3], dWx[1][3], Wy[1][3], dWy[1][3], Wz[1][3], dWz[1][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Wx[0][k] = X[0][k]; dWx[0][k] = dX[0][k];
+            Wy[0][k] = Y[0][k]; dWy[0][k] = dY[0][k];
+            Wz[0][k] = Z[0][k]; dWz[0][k] = dZ[0][k];
+        }
+        auto one = [](int, int, int) { return 1.0f; };
+        adj_position<1, 1, false>(Wx, dWx, Wy, dWy, Wz, dWz, lm, one, Mx, My, Mz);
+    }
+    lx[0] = fmaf(mt, Dx + Mx, lx[0]);
+    lx[1] = fmaf(mt, Dy + My, lx[1]);
+    lx[2] = fmaf(mt, Dz + Mz, lx[2]);
 }
 
 // With 27 modes, tiles of at most this many particles are walked in memory order
@@ -514,8 +532,8 @@ __device__ __forceinline__ void list_in_memory_order(const uint32_t *__restrict_
     __syncthreads();
 }
 
-template <int R>
-__global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas(R)) k_p2g_adjoint(AdjP2GArgs Q) {
+template <int R, bool FEW>
+__global__ void __launch_bounds__(kAdjThreads, p2g_adj_ctas<R, FEW>()) k_p2g_adjoint(AdjP2GArgs Q) {
     extern __shared__ float s_adj[];
     constexpr bool kList = R == 27;
     __shared__ uint32_t s_idx[kList ? kAdjList : 1], s_bits[kList ? 2 * kAdjWords + 1 : 1];
@@ -610,9 +628,10 @@ size_t adjoint_scratch_bytes(int64_t count) {
 template <int R>
 static cudaError_t launch_g2p_adjoint(const AdjG2PArgs &G, int64_t tiles, cudaStream_t s) {
     constexpr int smem = stage_bytes<R>();
-    const cudaError_t e = cudaFuncSetAttribute(k_g2p_adjoint<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const auto kernel = adj_few(R, G.count, tiles) ? k_g2p_adjoint<R, true> : k_g2p_adjoint<R, false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_g2p_adjoint<R><<<(int)tiles, kAdjThreads, smem, s>>>(G);
+    kernel<<<(int)tiles, kAdjThreads, smem, s>>>(G);
     return cudaGetLastError();
 }
 
@@ -622,9 +641,11 @@ static cudaError_t launch_p2g_adjoint(const AdjP2GArgs &Q, int64_t tiles, cudaSt
     constexpr int limit = tiles_bytes + 2 * stage_bytes<R>();  // the kernel's, whatever the call
     static_assert(limit <= 200 * 1024, "the P2G adjoint exceeds the shared memory of a CTA");
     const int smem = tiles_bytes + (Q.accumulate ? 2 : 1) * stage_bytes<R>();
-    const cudaError_t e = cudaFuncSetAttribute(k_p2g_adjoint<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+    const bool few = R == 27 || adj_few(R, Q.count, tiles);
+    const auto kernel = few ? k_p2g_adjoint<R, true> : k_p2g_adjoint<R, R == 27>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
-    k_p2g_adjoint<R><<<(int)tiles, kAdjThreads, smem, s>>>(Q);
+    kernel<<<(int)tiles, kAdjThreads, smem, s>>>(Q);
     return cudaGetLastError();
 }
 
