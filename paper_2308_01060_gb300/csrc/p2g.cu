@@ -300,8 +300,11 @@ cudaError_t p2g_reduce(const P2GArgs &P, float *gm[3], float *gp[3], bool accumu
     return reduce_tiles(P, gm, gp, nullptr, 0.0f, nullptr, accumulate, s);
 }
 
+// The movers of the fused transfer: a few per block (8% of the particles change
+// cell), where the chunk kernel has one chunk a block to hide its loads behind:
+// 27 modes, 0.3 million movers in 128^3, 354 us against 188.
 cudaError_t p2g_accumulate(const P2GArgs &P, float *gm[3], float *gp[3], int R, cudaStream_t s) {
-    const cudaError_t e = launch_p2g(P, R, POLYPIC_COEFF_F32, s);
+    const cudaError_t e = launch_tiles_f32(P, R, (int)(P.nblocks / kP2GWarps), s);
     if (e != cudaSuccess) return e;
     return reduce_tiles(P, gm, gp, nullptr, 0.0f, nullptr, true, s);
 }

@@ -1,5 +1,6 @@
-// p2g_tiles.cuh -- the lane-per-cell P2G kernel of 1, 4 and 8 modes (its
-// per-particle pieces are in p2g_kernel.cuh) and its launcher.  Each
+// p2g_tiles.cuh -- the lane-per-cell P2G kernel of 1, 4 and 8 modes, and of the
+// fused transfer's movers (its per-particle pieces are in p2g_kernel.cuh), and
+// its launcher.  Each
 // instantiation is compiled in one of the p2g_tiles_*.cu translation units.
 //
 // Work decomposition (no float atomics, bit-identical from run to run): one
@@ -180,8 +181,8 @@ __device__ __forceinline__ void merge_tile(const float *smem_regions, const bool
 }
 
 template <int R, int FMT, bool ADJ, bool AFF>
-// two CTAs per SM fit without spills
-__global__ void __launch_bounds__(kP2GWarps * 32, 2)
+// two CTAs per SM fit without spills, but with 27 modes (one measured faster)
+__global__ void __launch_bounds__(kP2GWarps * 32, R == 27 ? 1 : 2)
     k_p2g_tiles(P2GArgs P) {
     extern __shared__ float smem[];
     __shared__ bool s_empty[kP2GWarps];

@@ -7,6 +7,7 @@ cudaError_t launch_tiles_f32(const P2GArgs &P, int R, int grid, cudaStream_t s) 
     if (R == 1) return launch_tiles<1, POLYPIC_COEFF_F32, false>(P, grid, s);
     if (R == 4) return launch_tiles<4, POLYPIC_COEFF_F32, false>(P, grid, s);
     if (R == 8) return launch_tiles<8, POLYPIC_COEFF_F32, false>(P, grid, s);
+    if (R == 27) return launch_tiles<27, POLYPIC_COEFF_F32, false>(P, grid, s);
     return cudaErrorInvalidValue;
 }
 
