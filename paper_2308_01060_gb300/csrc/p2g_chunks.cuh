@@ -85,10 +85,9 @@ template <int R, int FMT, bool ADJ, bool AFF, int G> constexpr int chunks_smem_b
 // weight is in Gp, Fu padded along A to 4 nodes (node = k + shift).
 template <int R> struct Contraction {
     static constexpr int D = axis_degrees(R);
-    static constexpr bool kPack = R >= 8;
     // after the contraction along w: [dv][kw], du = 0, 1 as a packed pair
     float2 p[D][3];
-    float s[D][3];  // du = 2 (27 modes); du = 0 for one mode
+    float s[D][3];  // du = 2 (27 modes)
 };
 
 template <int R, int A, class C>
@@ -97,41 +96,35 @@ __device__ __forceinline__ void contract_w(const C &coef, const float (&Fw)[axis
     constexpr int D = axis_degrees(R);
 #pragma unroll
     for (int dv = 0; dv < D; ++dv) {
-        if constexpr (D == 1) {
-            const float c = coef(0);
 #pragma unroll
-            for (int kw = 0; kw < 3; ++kw) T.s[dv][kw] = c * Fw[0][kw];
-        } else {
+        for (int kw = 0; kw < 3; ++kw) T.p[dv][kw] = make_float2(0.0f, 0.0f);
+        // du = 0, 1 packed: the pair's coefficients sit in neighbouring
+        // registers, only the axis factor is broadcast
 #pragma unroll
-            for (int kw = 0; kw < 3; ++kw) T.p[dv][kw] = make_float2(0.0f, 0.0f);
-            // du = 0, 1 packed: the pair's coefficients sit in neighbouring
-            // registers, only the axis factor is broadcast
+        for (int dw = 0; dw < D; ++dw) {
+            const bool h0 = has_mode(R, deg_x<A>(0, dv, dw), deg_y<A>(0, dv, dw), deg_z<A>(0, dv, dw));
+            const bool h1 = has_mode(R, deg_x<A>(1, dv, dw), deg_y<A>(1, dv, dw), deg_z<A>(1, dv, dw));
+            if (h0 && h1) {
+                const float2 c = make_float2(
+                    coef(mode_index(deg_x<A>(0, dv, dw), deg_y<A>(0, dv, dw), deg_z<A>(0, dv, dw))),
+                    coef(mode_index(deg_x<A>(1, dv, dw), deg_y<A>(1, dv, dw), deg_z<A>(1, dv, dw))));
 #pragma unroll
-            for (int dw = 0; dw < D; ++dw) {
-                const bool h0 = has_mode(R, deg_x<A>(0, dv, dw), deg_y<A>(0, dv, dw), deg_z<A>(0, dv, dw));
-                const bool h1 = has_mode(R, deg_x<A>(1, dv, dw), deg_y<A>(1, dv, dw), deg_z<A>(1, dv, dw));
-                if (h0 && h1) {
-                    const float2 c = make_float2(
-                        coef(mode_index(deg_x<A>(0, dv, dw), deg_y<A>(0, dv, dw), deg_z<A>(0, dv, dw))),
-                        coef(mode_index(deg_x<A>(1, dv, dw), deg_y<A>(1, dv, dw), deg_z<A>(1, dv, dw))));
+                for (int kw = 0; kw < 3; ++kw)
+                    T.p[dv][kw] = dw == 0 ? __fmul2_rn(c, bcast(Fw[dw][kw]))
+                                          : __ffma2_rn(c, bcast(Fw[dw][kw]), T.p[dv][kw]);
+            } else if (h0) {  // 4 modes: no product modes
+                const float c = coef(mode_index(deg_x<A>(0, dv, dw), deg_y<A>(0, dv, dw), deg_z<A>(0, dv, dw)));
 #pragma unroll
-                    for (int kw = 0; kw < 3; ++kw)
-                        T.p[dv][kw] = dw == 0 ? __fmul2_rn(c, bcast(Fw[dw][kw]))
-                                              : __ffma2_rn(c, bcast(Fw[dw][kw]), T.p[dv][kw]);
-                } else if (h0) {  // 4 modes: no product modes
-                    const float c = coef(mode_index(deg_x<A>(0, dv, dw), deg_y<A>(0, dv, dw), deg_z<A>(0, dv, dw)));
-#pragma unroll
-                    for (int kw = 0; kw < 3; ++kw) T.p[dv][kw].x = fmaf(c, Fw[dw][kw], T.p[dv][kw].x);
-                }
+                for (int kw = 0; kw < 3; ++kw) T.p[dv][kw].x = fmaf(c, Fw[dw][kw], T.p[dv][kw].x);
             }
-            if constexpr (D == 3) {
+        }
+        if constexpr (D == 3) {
 #pragma unroll
-                for (int dw = 0; dw < 3; ++dw) {
-                    const float c = coef(mode_index(deg_x<A>(2, dv, dw), deg_y<A>(2, dv, dw), deg_z<A>(2, dv, dw)));
+            for (int dw = 0; dw < 3; ++dw) {
+                const float c = coef(mode_index(deg_x<A>(2, dv, dw), deg_y<A>(2, dv, dw), deg_z<A>(2, dv, dw)));
 #pragma unroll
-                    for (int kw = 0; kw < 3; ++kw)
-                        T.s[dv][kw] = dw == 0 ? c * Fw[dw][kw] : fmaf(c, Fw[dw][kw], T.s[dv][kw]);
-                }
+                for (int kw = 0; kw < 3; ++kw)
+                    T.s[dv][kw] = dw == 0 ? c * Fw[dw][kw] : fmaf(c, Fw[dw][kw], T.s[dv][kw]);
             }
         }
     }
@@ -144,38 +137,30 @@ __device__ __forceinline__ float4 contract_column(const Contraction<R> &T,
                                                   const float2 (&Gp)[axis_degrees(R)][2], int kv,
                                                   int kw) {
     constexpr int D = axis_degrees(R);
-    float2 a, b;
-    if constexpr (D == 1) {
-        const float t = T.s[0][kw] * Fv[0][kv];
-        a = __fmul2_rn(bcast(t), Gp[0][0]);
-        b = __fmul2_rn(bcast(t), Gp[0][1]);
+    float2 t = __fmul2_rn(T.p[0][kw], bcast(Fv[0][kv]));
+    if constexpr (R == 4) {  // only du = 0 has a mode with dv = 1
+        t.x = fmaf(T.p[1][kw].x, Fv[1][kv], t.x);
     } else {
-        float2 t = __fmul2_rn(T.p[0][kw], bcast(Fv[0][kv]));
-        if constexpr (R == 4) {  // only du = 0 has a mode with dv = 1
-            t.x = fmaf(T.p[1][kw].x, Fv[1][kv], t.x);
-        } else {
 #pragma unroll
-            for (int dv = 1; dv < D; ++dv) t = __ffma2_rn(T.p[dv][kw], bcast(Fv[dv][kv]), t);
-        }
-        a = __fmul2_rn(bcast(t.x), Gp[0][0]);
-        b = __fmul2_rn(bcast(t.x), Gp[0][1]);
-        a = __ffma2_rn(bcast(t.y), Gp[1][0], a);
-        b = __ffma2_rn(bcast(t.y), Gp[1][1], b);
-        if constexpr (D == 3) {
-            float u = T.s[0][kw] * Fv[0][kv];
-            u = fmaf(T.s[1][kw], Fv[1][kv], u);
-            u = fmaf(T.s[2][kw], Fv[2][kv], u);
-            a = __ffma2_rn(bcast(u), Gp[2][0], a);
-            b = __ffma2_rn(bcast(u), Gp[2][1], b);
-        }
+        for (int dv = 1; dv < D; ++dv) t = __ffma2_rn(T.p[dv][kw], bcast(Fv[dv][kv]), t);
+    }
+    float2 a = __fmul2_rn(bcast(t.x), Gp[0][0]), b = __fmul2_rn(bcast(t.x), Gp[0][1]);
+    a = __ffma2_rn(bcast(t.y), Gp[1][0], a);
+    b = __ffma2_rn(bcast(t.y), Gp[1][1], b);
+    if constexpr (D == 3) {
+        float u = T.s[0][kw] * Fv[0][kv];
+        u = fmaf(T.s[1][kw], Fv[1][kv], u);
+        u = fmaf(T.s[2][kw], Fv[2][kv], u);
+        a = __ffma2_rn(bcast(u), Gp[2][0], a);
+        b = __ffma2_rn(bcast(u), Gp[2][1], b);
     }
     return make_float4(a.x, a.y, b.x, b.y);
 }
 
 // Eq 12's affine map: M = (I + dt C)^-1 with C_ab = c_{a, 1+b} (the linear
 // modes of all three components; stage rows R.. hold the other two
-// components'), the identity when |det(I + dt C)| < 1e-6.  In role order: rows
-// and columns u, v, w (the inverse permutes with the matrix).
+// components').  In role order: rows and columns u, v, w (the inverse permutes
+// with the matrix).
 template <int R, int A>
 __device__ __forceinline__ void affine_inverse(const float *st, float dt,
                                                float (&M)[3][3]) {
@@ -188,27 +173,7 @@ __device__ __forceinline__ void affine_inverse(const float *st, float dt,
             const int row = a == 0 ? 1 + ax[b] : R + 3 * (a - 1) + ax[b];
             C[a][b] = fmaf(dt, st[row * 32], a == b ? 1.0f : 0.0f);
         }
-    const float m00 = C[1][1] * C[2][2] - C[1][2] * C[2][1];
-    const float m01 = C[0][2] * C[2][1] - C[0][1] * C[2][2];
-    const float m02 = C[0][1] * C[1][2] - C[0][2] * C[1][1];
-    const float m10 = C[1][2] * C[2][0] - C[1][0] * C[2][2];
-    const float m11 = C[0][0] * C[2][2] - C[0][2] * C[2][0];
-    const float m12 = C[0][2] * C[1][0] - C[0][0] * C[1][2];
-    const float m20 = C[1][0] * C[2][1] - C[1][1] * C[2][0];
-    const float m21 = C[0][1] * C[2][0] - C[0][0] * C[2][1];
-    const float m22 = C[0][0] * C[1][1] - C[0][1] * C[1][0];
-    const float det = C[0][0] * m00 + C[0][1] * m10 + C[0][2] * m20;
-    if (fabsf(det) < 1e-6f) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) M[a][b] = a == b ? 1.0f : 0.0f;
-        return;
-    }
-    const float id = 1.0f / det;
-    M[0][0] = m00 * id; M[0][1] = m01 * id; M[0][2] = m02 * id;
-    M[1][0] = m10 * id; M[1][1] = m11 * id; M[1][2] = m12 * id;
-    M[2][0] = m20 * id; M[2][1] = m21 * id; M[2][2] = m22 * id;
+    inverse_or_identity(C, M);
 }
 
 // 8 and 27 modes under the map are not separable per axis: every stencil node
@@ -285,6 +250,8 @@ struct Chunk {
 template <int R, int FMT, bool ADJ, bool AFF, int G>
 __device__ __forceinline__ void p2g_item(const P2GArgs &P, uint32_t tile, int g, int a, int lane,
                                          float *ex, float *st, float *reg) {
+    static_assert(R == 4 || R == 8 || R == 27, "one mode has no use for the exchange");
+    static_assert(!AFF || R > 4, "the affine map of 4 modes is separable: k_p2g_tiles");
     constexpr int D = axis_degrees(R);
     constexpr int NB = 8 / G;
     constexpr bool F32 = FMT == POLYPIC_COEFF_F32;
@@ -452,7 +419,7 @@ __device__ __forceinline__ void p2g_item(const P2GArgs &P, uint32_t tile, int g,
             stage(pn, slot_of(nxt));
             cp_async_commit();
         };
-        if constexpr (AFF && R > 4) {
+        if constexpr (AFF) {
             Mapped<R> E;
             if (a == 0) E.template load<0>(P, st);
             else if (a == 1) E.template load<1>(P, st);
@@ -477,22 +444,8 @@ __device__ __forceinline__ void p2g_item(const P2GArgs &P, uint32_t tile, int g,
             auto contract = [&](auto axis) {
                 constexpr int A = decltype(axis)::value;
                 // the coefficient of mode r (16-bit codes: the low or high half of
-                // word r / 2; the affine map of 4 modes turns the linear ones into M^T c)
-                float cl[3] = {0.0f, 0.0f, 0.0f};  // in x, y, z order
-                if constexpr (AFF && R == 4) {
-                    constexpr int ax[3] = {A, A == 0 ? 1 : 0, A == 2 ? 1 : 2};
-                    float M[3][3];
-                    affine_inverse<R, A>(st, P.map_dt, M);
-#pragma unroll
-                    for (int e = 0; e < 3; ++e)
-                        cl[ax[e]] = st[(1 + ax[0]) * 32] * M[0][e] +
-                                    st[(1 + ax[1]) * 32] * M[1][e] +
-                                    st[(1 + ax[2]) * 32] * M[2][e];
-                }
+                // word r / 2)
                 auto coef = [&](int r) {
-                    if constexpr (AFF && R == 4) {
-                        if (r >= 1) return cl[r - 1];
-                    }
                     if constexpr (F32) {
                         return st[r * 32];
                     } else {
@@ -593,7 +546,7 @@ __device__ __forceinline__ void p2g_item(const P2GArgs &P, uint32_t tile, int g,
                 if (more) {
                     const uint32_t k = (b0 + nxt.ib) * 32 + lane;
                     want0 = P.cell_start[k];
-        want1 = P.cell_start[k + 1];
+                    want1 = P.cell_start[k + 1];
                 }
             }
         }

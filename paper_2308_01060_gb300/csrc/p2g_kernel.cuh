@@ -160,21 +160,8 @@ __device__ __forceinline__ void fit_rows(const Stencil1D &s, bool guard, float i
     }
 }
 
-// Eq 12's affine map: M = (I + dt C)^-1 with C_ab = c_{a, 1+b} (the linear
-// modes of all three components, component A's own row from its staged
-// coefficients), the identity when |det(I + dt C)| < 1e-6.
-template <int R, int A>
-__device__ __forceinline__ void affine_inverse(const float *st, int lane, float dt,
-                                               float (&M)[3][3]) {
-    using S = Stage<R, true>;
-    float C[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int slot = a == A ? S::kC + 1 + b : S::kL + 3 * (a < A ? a : a - 1) + b;
-            C[a][b] = fmaf(dt, st[slot * 32 + lane], a == b ? 1.0f : 0.0f);
-        }
+// M = C^-1, the identity when |det C| < 1e-6 (Eq 12's affine map: C = I + dt C_p).
+__device__ __forceinline__ void inverse_or_identity(const float (&C)[3][3], float (&M)[3][3]) {
     const float m00 = C[1][1] * C[2][2] - C[1][2] * C[2][1];
     const float m01 = C[0][2] * C[2][1] - C[0][1] * C[2][2];
     const float m02 = C[0][1] * C[1][2] - C[0][2] * C[1][1];
@@ -196,6 +183,24 @@ __device__ __forceinline__ void affine_inverse(const float *st, int lane, float 
     M[0][0] = m00 * id; M[0][1] = m01 * id; M[0][2] = m02 * id;
     M[1][0] = m10 * id; M[1][1] = m11 * id; M[1][2] = m12 * id;
     M[2][0] = m20 * id; M[2][1] = m21 * id; M[2][2] = m22 * id;
+}
+
+// Eq 12's affine map: M = (I + dt C)^-1 with C_ab = c_{a, 1+b} (the linear
+// modes of all three components, component A's own row from its staged
+// coefficients).
+template <int R, int A>
+__device__ __forceinline__ void affine_inverse(const float *st, int lane, float dt,
+                                               float (&M)[3][3]) {
+    using S = Stage<R, true>;
+    float C[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int slot = a == A ? S::kC + 1 + b : S::kL + 3 * (a < A ? a : a - 1) + b;
+            C[a][b] = fmaf(dt, st[slot * 32 + lane], a == b ? 1.0f : 0.0f);
+        }
+    inverse_or_identity(C, M);
 }
 
 // The 4-mode set under the map: sum_r c_r s_r(M z) = c_0 + sum_g (sum_b
