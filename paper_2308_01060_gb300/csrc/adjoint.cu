@@ -32,13 +32,13 @@ constexpr int kAdjThreads = 256;
 // CTAs of an SM that a gather's registers are limited for.  A phase of at most
 // one tile an SM (2048 particles each at 8 a cell) has no use for a second CTA,
 // only for the registers: on 119 thousand particles (33x29x45 cells) the P2G
-// adjoint of 8 modes takes 44 us with one and 53 with two, of 4 modes 37 and 47,
+// adjoint of 8 modes takes 45 us with one and 53 with two, of 4 modes 38 and 47,
 // the G2P adjoint with its scatter of 27 modes 97 and 111.  Larger phases take
-// two (863 thousand particles: P2G adjoint of 8 modes 121 us, 157 with one; G2P
+// two (863 thousand particles: P2G adjoint of 8 modes 124 us, 157 with one; G2P
 // adjoint of 27 modes 307, 319 with one), but for the P2G adjoint of 27 modes,
 // which would spill 376 bytes a thread (262 -> 275 us).  One mode is small
 // enough for two and, above two tiles an SM, three (2.9 million particles: P2G
-// adjoint 210 -> 177 us; 364 thousand: 39 us with two, 51 with three).  A sparse
+// adjoint 210 -> 184 us; 364 thousand: 39 us with two, 51 with three).  A sparse
 // phase has more tiles than its count says, so the grid's count as well (62
 // thousand particles in half of 64^3, G2P adjoint of 27 modes: 133 us with one,
 // 121 with two; grids up to 48^3 are below the line).
@@ -438,6 +438,19 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     const int64_t cnt = Q.count;
     float *__restrict__ cout = Q.out_c + (int64_t)A * R * cnt + p;
     float Dx = 0.0f, Dy = 0.0f, Dz = 0.0f;
+    {  // position terms of the mass, through the weights
+        float lm[3][3][3];
+        read_stencil<A>(tile_m, lx0, ly0, lz0, lm);
+        float Wx[1][3], dWx[1][3], Wy[1][3], dWy[1][3], Wz[1][3], dWz[1][3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Wx[0][k] = X[0][k]; dWx[0][k] = dX[0][k];
+            Wy[0][k] = Y[0][k]; dWy[0][k] = dY[0][k];
+            Wz[0][k] = Z[0][k]; dWz[0][k] = dZ[0][k];
+        }
+        auto one = [](int, int, int) { return 1.0f; };
+        adj_position<1, 1, false>(Wx, dWx, Wy, dWy, Wz, dWz, lm, one, Dx, Dy, Dz);
+    }
     float lmv[3][3][3];
     read_stencil<A>(tile_v, lx0, ly0, lz0, lmv);
     contract_modes<R, D>(X, Y, Z, lmv, [&](int a, const float (&m)[D][D]) {
@@ -451,25 +464,9 @@ __device__ __forceinline__ void p2g_adj_component(const AdjP2GArgs &Q, const Par
     });
     // position terms of the momentum, through the modes
     adj_position<R, D, false>(X, dX, Y, dY, Z, dZ, lmv, coef, Dx, Dy, Dz);
-    // position terms of the mass, through the weights (ahead of the momentum's:
-    // 1-5% slower), summed by themselves
-    float Mx = 0.0f, My = 0.0f, Mz = 0.0f;
-    {
-        float lm[3][3][3];
-        read_stencil<A>(tile_m, lx0, ly0, lz0, lm);
-        float Wx[1][3], dWx[1][3], Wy[1][3], dWy[1][3], Wz[1][3], dWz[1][3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            Wx[0][k] = X[0][k]; dWx[0][k] = dX[0][k];
-            Wy[0][k] = Y[0][k]; dWy[0][k] = dY[0][k];
-            Wz[0][k] = Z[0][k]; dWz[0][k] = dZ[0][k];
-        }
-        auto one = [](int, int, int) { return 1.0f; };
-        adj_position<1, 1, false>(Wx, dWx, Wy, dWy, Wz, dWz, lm, one, Mx, My, Mz);
-    }
-    lx[0] = fmaf(mt, Dx + Mx, lx[0]);
-    lx[1] = fmaf(mt, Dy + My, lx[1]);
-    lx[2] = fmaf(mt, Dz + Mz, lx[2]);
+    lx[0] = fmaf(mt, Dx, lx[0]);
+    lx[1] = fmaf(mt, Dy, lx[1]);
+    lx[2] = fmaf(mt, Dz, lx[2]);
 }
 
 // With 27 modes, tiles of at most this many particles are walked in memory order
