@@ -265,9 +265,13 @@ static cudaError_t reduce_tiles(const P2GArgs &P, float *gm[3], float *gp[3], fl
 // kernel, whose contraction keeps every lane busy; 1, 4 and 8 modes of a fluid
 // have too little contraction to pay for its exchange buffer: 460 us against
 // 372 (4 modes FP32) and 328 against 268 (8 modes FP16) on the fluids of 3.8
-// and 2.6 million particles, where 27 modes FP32 take 674 instead of 855.
-// These are spread fluids, cells filled unevenly; on freshly seeded ones (close
-// to 8 in every cell) 27 modes lose some 90 us by it, but no call knows that.
+// and 2.6 million particles, where 27 modes FP32 take 697 instead of 856.
+// These are spread fluids, cells filled unevenly.  What the chunk kernel loses by,
+// and no call knows of: cells filled evenly (close to 8 in every cell, as seeded;
+// P2G calls of 27 modes 45 -> 54 us on 33x29x45, 1.00 -> 1.06 ms on 7.6 million
+// particles) and phases of a particle a cell or fewer, one short chunk a block
+// (half of 128^3: 1 a cell 642 -> 689 us, 0.5 a cell 543 -> 662, solids of 8
+// modes 365 -> 487; at 2 a cell it wins, 807 -> 692 and 825 -> 518).
 static cudaError_t launch_p2g(const P2GArgs &P, int R, int fmt, cudaStream_t s) {
     const int grid = (int)(P.nblocks / kP2GWarps);
     if (P.affine) {  // Eq 12's affine map: FP32 coefficients, 4, 8 or 27 modes

@@ -26,11 +26,15 @@
 // footprint) and the shared-memory exchange, ~890 instructions a chunk and
 // face grid at 40% issue.  Two choices were worth more than any other:
 //   * the face grid is a run-time value, so that the SM's warps share one
-//     code: three unrolled copies missed the instruction cache (891 -> 674 us
-//     on 3.8 million particles, 27 modes FP32);
-//   * the shared memory of an SM stays under the 164 KB carve-out: L1 holds the
-//     lines of the loads in flight, and the next step up (60 KB of L1 instead
-//     of 92) cost 10%, two stages of coefficients (28 KB) 50%.
+//     code: three unrolled copies missed the instruction cache (891 us against
+//     674 in the runs that compared them, 3.8 million particles, 27 modes FP32);
+//   * L1 holds the lines of the loads in flight: the two CTAs of 27 modes FP32
+//     of a fluid, and of the 16-bit formats, stay under the 164 KB carve-out of
+//     shared memory by 384 bytes and more; the next step up (60 KB of L1 instead
+//     of 92) cost 10%, two stages of coefficients (28 KB) 50%.  With two groups
+//     a solid phase's absorbed mass and the affine map's six words take them
+//     above it.
+// In the form kept, P2G of those 3.8 million takes 697 us (lane per cell: 856).
 #pragma once
 #include <type_traits>
 
@@ -626,9 +630,11 @@ cudaError_t launch_chunks_g(const P2GArgs &P, int grid, cudaStream_t s) {
 // Two groups (two CTAs of 6 warps on an SM) overlap one tile's prologue and
 // merge with the other's work; four groups (one CTA of 12) give a tile twice the
 // warps.  With fewer than about four tiles of 2048 particles per SM the last
-// wave decides: 4 groups took 64 us instead of 93 (33x29x45 cells, 119
-// thousand particles, 27 modes) and 204 instead of 212 (64^3, 863 thousand); on
-// 128^3 and 3.8 million 2 groups took 741 instead of 781.
+// wave decides: the P2G call takes 62 us with 4 groups and 92 with 2 (33x29x45
+// cells, 119 thousand particles, 27 modes), 200 and 210 (64^3, 863 thousand); on
+// 128^3 and 3.8 million the kernel takes 697 us with 2 and 729 with 4.  A sparse
+// phase has more tiles than its count says (half of 128^3 with 0.5 million: 661
+// us with 4, 539 with 2); no call knows that.
 constexpr int64_t kWideTiles = 152 * 4 * 2048;
 template <int R, int FMT, bool ADJ, bool AFF = false>
 cudaError_t launch_chunks(const P2GArgs &P, int grid, cudaStream_t s) {

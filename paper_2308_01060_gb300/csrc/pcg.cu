@@ -27,7 +27,7 @@
 // all smaller levels run in one CTA from shared memory.  The working set stays in L2
 // (60 MB at 128^3); a pass is bound by its loads' latency and by launching.
 // The grid update of 128^3 with 476 thousand fluid cells, 24 iterations, takes
-// 2.09 ms; 4.68 ms before, with a thread per cell of the box on every level,
+// 1.97 ms; 4.68 ms before, with a thread per cell of the box on every level,
 // 23 launches per iteration and the coarsest level's operator read from memory
 // on each of its 32 sweeps.
 #include <algorithm>
@@ -126,8 +126,9 @@ constexpr int kMgMaxLevels = 12;
 constexpr int kMgCoarsest = 512;      // cells of the level swept in one CTA
 constexpr int kMgCoarseSweeps = 32;
 constexpr float kMgOmega = 2.0f / 3.0f;
-// Levels of at most this many cells run in one CTA (16^3 fits; the shared
-// memory of it and the levels below bounds it).
+// Levels of at most this many cells run in one CTA (16^3 fits): a thread keeps
+// the operator of its five cells of the first one in registers, 64 of them at
+// 1024 threads (the shared memory would hold more).
 constexpr int64_t kMgSmall = 4608;
 constexpr int kMgSmallThreads = 1024;
 // All the shared memory a CTA can have.  The levels of 128^3 take 64 KB, no
